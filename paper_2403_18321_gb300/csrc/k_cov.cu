@@ -18,15 +18,46 @@ namespace gbpca {
 
 namespace {
 
-constexpr int kSyrkThreads = 256;
-constexpr int kChunk = 32;  // pixels staged in shared memory per iteration
+// Threads of a CTA at most; a slot's tiles take as many CTAs as they need, two
+// or more of which share an SM, so that one's loads run beside the others'
+// products.  FP64: the pipe is so slow that what counts is how often the CTAs
+// of a slot repeat the conversion of its pixels.
+template <typename Acc>
+constexpr int max_threads() { return sizeof(Acc) == 8 ? 384 : 256; }
+// Columns of a thread's tile (rows: TM = 8 in FP32, 4 in FP64): 8 x 4 rather than
+// 8 x 8 gives a slot of 103 bands 6 warps instead of 3, and the SMs hold few slots.
+template <typename Acc>
+constexpr int tile_cols() { return 4; }
+constexpr int kChunk = 32;  // pixels whose band sums are added in the accumulator's type before FP64
+constexpr int kStage = 16;  // pixels staged in shared memory at a time
+constexpr int kAhead = 4;   // raw stages: a stage's products take less time than its copy
 
 template <typename In>
 __device__ __forceinline__ float ld(const In* p) { return to_f32<In>(*p); }
 
+// Asynchronous copy of a 16-byte unit, of which `bytes` exist.
+__device__ __forceinline__ void copy_unit(uint32_t dst, const void* src, int bytes) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes)
+               : "memory");
+}
+// 16-byte units of a raw stage: kStage pixels, one more for a start between units.
+__host__ __device__ inline int raw_units(int B, int el) { return (kStage * B * el + 15) / 16 + 1; }
+
 // One CTA: pixels [n0, n1) of the cube into partial slot g (S1 when grp is
-// 0), band-tile group grp.  Each thread owns one TM x TM tile of the upper
-// block-triangle of S2.
+// 0), band-tile group grp.  Each thread owns one TM x TN tile of the upper
+// block-triangle of S2 and adds its products pixel by pixel.
+//
+// Bound: the FP32 (FP64) pipe.  The pixels come in by asynchronous copies, one
+// stage ahead, and are centred once per CTA into a second buffer (loads into
+// registers, a few at a time between two barriers, took 14 of every 15 us).
+// Tile t holds TM / U units of U consecutive bands (16 bytes), unit u being
+// bands u Bu + U t and on, so that the lanes of a warp -- consecutive tiles of
+// a row of tiles -- read consecutive 16-byte words of a pixel.
+// A slot's 8 x 4 tiles give the few slots an SM holds (two or three) enough warps.
+// 610 x 340 x 103 FP32, the whole covariance call: 391 us with 8 x 8 tiles of
+// consecutive bands and synchronous loads, 231 us with the copies, 213 us with
+// the smaller tiles.  350 x 350 x 188 in FP64 (two CTAs an SM): the fit 6.38 -> 6.15
+// ms, of which the FP64 pipe at its full rate takes 3.6.
 template <typename In, typename Acc, int TM>
 __device__ __forceinline__ void syrk_simt_cta(const In* __restrict__ cube, int B, int64_t n0,
                                               int64_t n1, int g, int grp,
@@ -34,78 +65,140 @@ __device__ __forceinline__ void syrk_simt_cta(const In* __restrict__ cube, int B
                                               double* __restrict__ s1_part,
                                               Acc* __restrict__ s2_part,
                                               int* __restrict__ escale, unsigned char* smem_raw) {
-  const int Bt = (B + TM - 1) / TM, ntiles = Bt * (Bt + 1) / 2;
+  constexpr int U = 16 / (int)sizeof(Acc), NU = TM / U;   // bands per unit, units per row tile
+  constexpr int TN = tile_cols<Acc>(), NC = TN / U, HV = NU / NC;   // column units; column parts
+  struct __align__(16) Unit { Acc v[U]; };
+  const int Bt = (B + TM - 1) / TM, ntiles = HV * Bt * (Bt + 1) / 2;
   const int s2_elems = B * (B + 1) / 2;
-  const int Bpad = Bt * TM;
-  Acc* xs = reinterpret_cast<Acc*>(smem_raw);                   // [kChunk][Bpad]
-  float* sh = reinterpret_cast<float*>(xs + kChunk * Bpad);     // [Bpad] shift
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int Bpad = Bt * TM, Bu = Bt * U;                  // unit u of tile t: bands u Bu + U t ..
+  Acc* xs = reinterpret_cast<Acc*>(smem_raw);                   // [kStage][Bpad]
+  float* sh = reinterpret_cast<float*>(xs + kStage * Bpad);     // [Bpad] shift
+  float4* raw = reinterpret_cast<float4*>(sh + ((Bpad + 3) & ~3));   // [kAhead][raw_units]
+  const int ru = raw_units(B, (int)sizeof(In));
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nthr = blockDim.x;
 
-  for (int b = tid; b < Bpad; b += kSyrkThreads) sh[b] = b < B ? ld(cube + b) : 0.f;
+  for (int b = tid; b < Bpad; b += nthr) sh[b] = b < B ? ld(cube + b) : 0.f;
   if (g == 0 && grp == 0)
-    for (int b = tid; b < B; b += kSyrkThreads) {
+    for (int b = tid; b < B; b += nthr) {
       shift_out[b] = ld(cube + b);
       if (escale != nullptr) escale[b] = 0;
     }
 
-  // tile of this thread: enumerate the upper block-triangle row by row
-  const int t = grp * kSyrkThreads + tid;
-  int ti = -1, tj = -1;
+  // tile of this thread: enumerate the upper block-triangle row by row, a row's
+  // column parts one after the other
+  const int t = grp * nthr + tid;
+  int ti = -1, tj = -1, part = 0;
   if (t < ntiles) {
     int rem = t;
     for (int r = 0; r < Bt; ++r) {
       const int len = Bt - r;
-      if (rem < len) { ti = r; tj = r + rem; break; }
-      rem -= len;
+      if (rem < HV * len) { ti = r; part = rem / len; tj = r + rem - part * len; break; }
+      rem -= HV * len;
     }
   }
-  Acc acc[TM][TM];
+  Acc acc[TM][TN];
 #pragma unroll
   for (int i = 0; i < TM; ++i)
 #pragma unroll
-    for (int j = 0; j < TM; ++j) acc[i][j] = Acc(0);
-  double s1 = 0.0;  // band `tid` (block-row 0 of the grid only)
-  __syncthreads();
+    for (int j = 0; j < TN; ++j) acc[i][j] = Acc(0);
+  double s1[2] = {0.0, 0.0};  // bands tid and tid + nthr (group 0 only; B <= 2 nthr)
+  Acc cs[2] = {Acc(0), Acc(0)};
+  // stage at pixel c: the whole 16-byte units that hold its values (the cube
+  // starts on one; the last one may end beyond the cube)
+  auto fetch = [&](int64_t c, int buf) {
+    const int cp = (int)((n1 - c) < kStage ? (n1 - c) : kStage);
+    const int64_t b0 = c * B * (int64_t)sizeof(In);
+    const int skip = (int)(b0 & 15), bytes = skip + cp * B * (int)sizeof(In);
+    const char* src = reinterpret_cast<const char*>(cube) + (b0 - skip);
+    const uint32_t dst = (uint32_t)__cvta_generic_to_shared(raw + buf * ru);
+    for (int u = tid * 16; u < bytes; u += nthr * 16)
+      copy_unit(dst + (uint32_t)u, src + u, bytes - u < 16 ? bytes - u : 16);
+  };
+  for (int k = 0; k < kAhead - 1; ++k) {
+    if (n0 + k * kStage < n1) fetch(n0 + k * kStage, k);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  }
 
-  for (int64_t c0 = n0; c0 < n1; c0 += kChunk) {
-    const int cp = (int)((n1 - c0) < kChunk ? (n1 - c0) : kChunk);
-    for (int p = warp; p < kChunk; p += kSyrkThreads / 32) {
-      const In* row = cube + (c0 + p) * (int64_t)B;
-      for (int b = lane; b < Bpad; b += 32)
-        xs[p * Bpad + b] = (p < cp && b < B) ? Acc(ld(row + b)) - Acc(sh[b]) : Acc(0);
-    }
-    __syncthreads();
-    if (grp == 0 && tid < B) {
-      Acc cs = Acc(0);
-      for (int p = 0; p < cp; ++p) cs += xs[p * Bpad + tid];
-      s1 += (double)cs;
-    }
-    if (ti >= 0) {
-      const Acc* xa = xs + ti * TM;
-      const Acc* xb = xs + tj * TM;
-      for (int p = 0; p < cp; ++p) {
-        Acc a[TM], bv[TM];
+  int buf = 0;
+  for (int64_t c0 = n0; c0 < n1; c0 += kStage, buf = (buf + 1) % kAhead) {
+    const int cp = (int)((n1 - c0) < kStage ? (n1 - c0) : kStage);
+    asm volatile("cp.async.wait_group %0;" ::"n"(kAhead - 2) : "memory");
+    __syncthreads();   // this stage has landed; the previous one's products are done
+    if (c0 + (kAhead - 1) * kStage < n1) fetch(c0 + (kAhead - 1) * kStage, (buf + kAhead - 1) % kAhead);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    const In* rp = reinterpret_cast<const In*>(raw + buf * ru) +
+                   (int)((c0 * B * (int64_t)sizeof(In)) & 15) / (int)sizeof(In);
+    const bool sum_done = ((c0 - n0) / kStage) % (kChunk / kStage) == kChunk / kStage - 1;
 #pragma unroll
-        for (int i = 0; i < TM; ++i) { a[i] = xa[p * Bpad + i]; bv[i] = xb[p * Bpad + i]; }
+    for (int h = 0; h < 2; ++h) {
+      const int b = tid + h * nthr;
+      if (b >= Bpad) continue;
+      const Acc sb = Acc(sh[b]);
+      const int bb = b < B ? b : 0;
+      Acc sum = cs[h];
+      constexpr int kV = sizeof(Acc) == 8 ? 4 : 16;   // values in flight
 #pragma unroll
-        for (int i = 0; i < TM; ++i)
+      for (int p0 = 0; p0 < kStage; p0 += kV) {
+        Acc v[kV];
 #pragma unroll
-          for (int j = 0; j < TM; ++j) acc[i][j] = fma(a[i], bv[j], acc[i][j]);
+        for (int p = 0; p < kV; ++p) v[p] = Acc(ld(rp + (p0 + p < cp ? p0 + p : 0) * B + bb)) - sb;
+#pragma unroll
+        for (int p = 0; p < kV; ++p) {
+          const bool in = p0 + p < cp && b < B;
+          xs[(p0 + p) * Bpad + b] = in ? v[p] : Acc(0);
+          if (in) sum += v[p];
+        }
+      }
+      cs[h] = sum;
+      if (sum_done || c0 + kStage >= n1) {
+        s1[h] += (double)sum;
+        cs[h] = Acc(0);
       }
     }
     __syncthreads();
+    if (ti >= 0) {
+      const Acc* xa = xs + ti * U;
+      const Acc* xb = xs + part * Bu + tj * U;
+#pragma unroll 2
+      for (int p = 0; p < cp; ++p) {
+        Acc a[TM], bv[TN];
+#pragma unroll
+        for (int u = 0; u < NU; ++u) {
+          const Unit x = *reinterpret_cast<const Unit*>(xa + p * Bpad + u * Bu);
+#pragma unroll
+          for (int i = 0; i < U; ++i) a[u * U + i] = x.v[i];
+        }
+#pragma unroll
+        for (int u = 0; u < NC; ++u) {
+          const Unit y = *reinterpret_cast<const Unit*>(xb + p * Bpad + u * Bu);
+#pragma unroll
+          for (int i = 0; i < U; ++i) bv[u * U + i] = y.v[i];
+        }
+#pragma unroll
+        for (int i = 0; i < TM; ++i)
+#pragma unroll
+          for (int j = 0; j < TN; ++j) acc[i][j] = fma(a[i], bv[j], acc[i][j]);
+      }
+    }
   }
+  __syncthreads();
 
-  if (grp == 0 && tid < B) s1_part[(size_t)g * B + tid] = s1;
+  if (grp == 0) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      if (tid + h * nthr < B) s1_part[(size_t)g * B + tid + h * nthr] = s1[h];
+  }
   if (ti >= 0) {
     Acc* out = s2_part + (size_t)g * s2_elems;
 #pragma unroll
     for (int i = 0; i < TM; ++i) {
-      const int r = ti * TM + i;
+      const int r = (i / U) * Bu + ti * U + i % U;
 #pragma unroll
-      for (int j = 0; j < TM; ++j) {
-        const int c = tj * TM + j;
-        if (r < B && c < B && r <= c) out[packed_index(r, c, B)] = acc[i][j];
+      for (int j = 0; j < TN; ++j) {
+        const int c = (part + j / U) * Bu + tj * U + j % U;
+        // the tiles of ti = tj form every pair twice
+        if (r < B && c < B && (ti != tj || r <= c))
+          out[r <= c ? packed_index(r, c, B) : packed_index(c, r, B)] = acc[i][j];
       }
     }
   }
@@ -116,7 +209,7 @@ __device__ __forceinline__ void syrk_simt_cta(const In* __restrict__ cube, int B
 // tensor-core pass) runs on a small grid that returns at once when the flag is
 // clear, instead of one CTA per slot.
 template <typename In, typename Acc, int TM, bool kGuarded>
-__global__ void __launch_bounds__(kSyrkThreads)
+__global__ void __launch_bounds__(max_threads<Acc>(), 2)
 k_syrk_simt(const In* __restrict__ cube, int64_t N, int B, int parts, float* __restrict__ shift_out,
             double* __restrict__ s1_part, Acc* __restrict__ s2_part,
             const int* __restrict__ guard, int* __restrict__ escale) {
@@ -141,20 +234,20 @@ k_syrk_simt(const In* __restrict__ cube, int64_t N, int B, int parts, float* __r
 // when none is set, so that the common case costs a few microseconds, not one
 // CTA per item.
 template <typename In, typename Acc, int TM, bool kGuarded>
-__global__ void __launch_bounds__(kSyrkThreads)
+__global__ void __launch_bounds__(max_threads<Acc>(), 2)
 k_syrk_simt_grouped(const TileDesc* __restrict__ T, const CovItem* __restrict__ items, int nitems,
                     int ntiles) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   if constexpr (kGuarded) {
     int any = 0;
-    for (int i = threadIdx.x; i < ntiles; i += kSyrkThreads)
+    for (int i = threadIdx.x; i < ntiles; i += blockDim.x)
       any |= *(volatile const int*)&T[i].hdr->cov_range;
     if (!__syncthreads_or(any)) return;
     for (int x = blockIdx.x; x < nitems; x += gridDim.x) {
       const CovItem it = items[x];
       const TileDesc& t = T[it.tile];
       const int B = t.B, Bt = (B + TM - 1) / TM;
-      if ((int)blockIdx.y * kSyrkThreads >= Bt * (Bt + 1) / 2) continue;
+      if ((int)(blockIdx.y * blockDim.x) >= TM / tile_cols<Acc>() * Bt * (Bt + 1) / 2) continue;
       if (*(volatile const int*)&t.hdr->cov_range == 0) continue;
       syrk_simt_cta<In, Acc, TM>(static_cast<const In*>(t.cube), B, it.p0, it.p1, it.slot,
                                  blockIdx.y, t.shift, t.s1p, static_cast<Acc*>(t.s2p), t.escale,
@@ -165,11 +258,19 @@ k_syrk_simt_grouped(const TileDesc* __restrict__ T, const CovItem* __restrict__ 
     const CovItem it = items[blockIdx.x];
     const TileDesc& t = T[it.tile];
     const int B = t.B, Bt = (B + TM - 1) / TM;
-    if ((int)blockIdx.y * kSyrkThreads >= Bt * (Bt + 1) / 2) return;
+    if ((int)(blockIdx.y * blockDim.x) >= TM / tile_cols<Acc>() * Bt * (Bt + 1) / 2) return;
     syrk_simt_cta<In, Acc, TM>(static_cast<const In*>(t.cube), B, it.p0, it.p1, it.slot,
                                blockIdx.y, t.shift, t.s1p, static_cast<Acc*>(t.s2p), nullptr,
                                smem_raw);
   }
+}
+
+// Threads and CTAs of a slot: the tiles in as few CTAs as hold them, evenly.
+template <typename Acc>
+void syrk_shape(int B, int TM, int* threads, int* groups) {
+  const int Bt = (B + TM - 1) / TM, n = TM / tile_cols<Acc>() * Bt * (Bt + 1) / 2;
+  *groups = (n + max_threads<Acc>() - 1) / max_threads<Acc>();
+  *threads = ((n + *groups - 1) / *groups + 31) & ~31;
 }
 
 template <typename In>
@@ -179,21 +280,25 @@ cudaError_t syrk_simt_typed(const In* cube, int64_t N, int B, bool fp64, float* 
   const int gx = guard != nullptr ? std::min(partials, 4 * device_sms()) : partials;
   if (fp64) {
     constexpr int TM = 4;
-    const int Bt = (B + TM - 1) / TM, ntiles = Bt * (Bt + 1) / 2;
-    const int groups = (ntiles + kSyrkThreads - 1) / kSyrkThreads;
-    const size_t smem = (size_t)kChunk * Bt * TM * sizeof(double) + Bt * TM * sizeof(float);
+    const int Bt = (B + TM - 1) / TM;
+    int threads, groups;
+    syrk_shape<double>(B, TM, &threads, &groups);
+    const size_t smem = (size_t)kStage * Bt * TM * sizeof(double) + Bt * TM * sizeof(float) +
+                        16 + kAhead * sizeof(float4) * (size_t)raw_units(Bt * TM, (int)sizeof(In));
     auto kern = guard != nullptr ? k_syrk_simt<In, double, TM, true> : k_syrk_simt<In, double, TM, false>;
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    kern<<<dim3(gx, groups), kSyrkThreads, smem, st>>>(cube, N, B, partials, shift, s1_part,
+    kern<<<dim3(gx, groups), threads, smem, st>>>(cube, N, B, partials, shift, s1_part,
                                                        (double*)s2_part, guard, escale);
   } else {
     constexpr int TM = 8;
-    const int Bt = (B + TM - 1) / TM, ntiles = Bt * (Bt + 1) / 2;
-    const int groups = (ntiles + kSyrkThreads - 1) / kSyrkThreads;
-    const size_t smem = (size_t)kChunk * Bt * TM * sizeof(float) + Bt * TM * sizeof(float);
+    const int Bt = (B + TM - 1) / TM;
+    int threads, groups;
+    syrk_shape<float>(B, TM, &threads, &groups);
+    const size_t smem = (size_t)kStage * Bt * TM * sizeof(float) + Bt * TM * sizeof(float) +
+                        16 + kAhead * sizeof(float4) * (size_t)raw_units(Bt * TM, (int)sizeof(In));
     auto kern = guard != nullptr ? k_syrk_simt<In, float, TM, true> : k_syrk_simt<In, float, TM, false>;
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    kern<<<dim3(gx, groups), kSyrkThreads, smem, st>>>(cube, N, B, partials, shift, s1_part,
+    kern<<<dim3(gx, groups), threads, smem, st>>>(cube, N, B, partials, shift, s1_part,
                                                        (float*)s2_part, guard, escale);
   }
   return cudaGetLastError();
@@ -206,22 +311,28 @@ cudaError_t syrk_simt_grouped_typed(const TileDesc* T, const CovItem* items, int
   const int gx = guarded ? std::min(nitems, 4 * device_sms()) : nitems;
   if (fp64) {
     constexpr int TM = 4;
-    const int Bt = (maxB + TM - 1) / TM, groups = (Bt * (Bt + 1) / 2 + kSyrkThreads - 1) / kSyrkThreads;
-    const size_t smem = (size_t)kChunk * Bt * TM * sizeof(double) + Bt * TM * sizeof(float);
+    const int Bt = (maxB + TM - 1) / TM;
+    int threads, groups;
+    syrk_shape<double>(maxB, TM, &threads, &groups);
+    const size_t smem = (size_t)kStage * Bt * TM * sizeof(double) + Bt * TM * sizeof(float) +
+                        16 + kAhead * sizeof(float4) * (size_t)raw_units(Bt * TM, (int)sizeof(In));
     auto kern = guarded ? k_syrk_simt_grouped<In, double, TM, true>
                         : k_syrk_simt_grouped<In, double, TM, false>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    kern<<<dim3(gx, groups), kSyrkThreads, smem, st>>>(T, items, nitems, ntiles);
+    kern<<<dim3(gx, groups), threads, smem, st>>>(T, items, nitems, ntiles);
   } else {
     constexpr int TM = 8;
-    const int Bt = (maxB + TM - 1) / TM, groups = (Bt * (Bt + 1) / 2 + kSyrkThreads - 1) / kSyrkThreads;
-    const size_t smem = (size_t)kChunk * Bt * TM * sizeof(float) + Bt * TM * sizeof(float);
+    const int Bt = (maxB + TM - 1) / TM;
+    int threads, groups;
+    syrk_shape<float>(maxB, TM, &threads, &groups);
+    const size_t smem = (size_t)kStage * Bt * TM * sizeof(float) + Bt * TM * sizeof(float) +
+                        16 + kAhead * sizeof(float4) * (size_t)raw_units(Bt * TM, (int)sizeof(In));
     auto kern = guarded ? k_syrk_simt_grouped<In, float, TM, true>
                         : k_syrk_simt_grouped<In, float, TM, false>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    kern<<<dim3(gx, groups), kSyrkThreads, smem, st>>>(T, items, nitems, ntiles);
+    kern<<<dim3(gx, groups), threads, smem, st>>>(T, items, nitems, ntiles);
   }
   return cudaGetLastError();
 }
