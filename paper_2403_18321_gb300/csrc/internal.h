@@ -180,9 +180,8 @@ cudaError_t launch_cov_finalize(const float* shift, const double* s1_part, const
                                 double* C, float* mu_f, double* dvec, DevHeader* hdr,
                                 cudaStream_t st, const int* escale = nullptr);
 
-// FP32 odd-even Jacobi on one thread-block cluster (matrix rows split over
-// the CTAs, rows of V in registers): writes diag32 [B'] and V32 [B'][B'].
-// relative_stop selects the element-wise relative stop test (else
+// FP32 odd-even Jacobi on one thread-block cluster: writes diag32 [B'] and V32
+// [B'][B'].  relative_stop selects the element-wise relative stop test (else
 // off(A) <= tol ||A||_F).
 cudaError_t launch_jacobi_cluster(const double* C, int B, float tol32, int sweeps_max,
                                   bool relative_stop, float* diag32, float* v32, DevHeader* hdr,
@@ -295,21 +294,25 @@ cudaError_t launch_cov_finalize_batched(const TileDesc* T, int ntiles, int maxB,
                                         bool escaled, cudaStream_t st);
 // Jacobi parameter lists: matrices of one shape (equal V width and cluster
 // size) run in one launch, one cluster each.
-int jacobi_width(int B);     // V values per lane of a V row (kernel variant)
-int jacobi_min_ctas(int B);  // fewest CTAs per cluster of the default kernel variant
-int jacobi_batch_ctas(int B);  // fewest CTAs per cluster of any variant (batched form)
-// The fewest CTAs, at least n, whose cluster holds a matrix of B bands (some
-// variant fits); n <= 0 gives jacobi_batch_ctas(B).
+int jacobi_width(int B);     // kernel variant: matrices of one variant and cluster size share a launch
+// The fewest CTAs, at least n, whose cluster holds a matrix of B bands.
 int jacobi_ctas_at_least(int B, int n);
+constexpr int kJacobiParamsBytes = 128;
 size_t jacobi_params_bytes();
-// Writes the parameters of one matrix to dst (host) for a cluster of nA CTAs
+// Writes the parameters of one matrix to dst (host) for a cluster of n CTAs
 // (0: the latency-oriented default of the single-matrix form); returns the
 // dynamic shared memory its cluster needs.
 size_t jacobi_fill_params(void* dst, const double* C, int B, float tol32, int sweeps_max,
-                          bool relative_stop, float* diag32, float* v32, DevHeader* hdr, int nA);
-int jacobi_params_ctas(const void* params);
+                          bool relative_stop, float* diag32, float* v32, DevHeader* hdr, int n);
 cudaError_t launch_jacobi_cluster_list(const void* host_first, const void* dev_list, int count,
                                        size_t smem, cudaStream_t st);
+// The matrix in one SM's shared memory (up to 128 bands).
+bool jacobi_sm_supported(int B);
+int jacobi_sm_fewest(int B);   // CTAs: the matrix's and the fewest that hold V
+size_t jacobi_sm_fill(void* dst, const double* C, int B, float tol32, int sweeps_max,
+                         bool relative_stop, float* diag32, float* v32, DevHeader* hdr, int n);
+cudaError_t launch_jacobi_sm(const void* host_first, const void* dev_list, int count, size_t smem,
+                                cudaStream_t st);
 cudaError_t launch_compact_batched(const TileDesc* T, int ntiles, int maxB, cudaStream_t st);
 cudaError_t launch_to_df_batched(const TileDesc* T, int ntiles, int maxB, cudaStream_t st);
 // One refinement iteration / orthogonalisation step of every tile; `flip`

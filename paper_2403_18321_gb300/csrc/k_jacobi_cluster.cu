@@ -1,5 +1,6 @@
 // k_jacobi_cluster.cu -- the cyclic Jacobi eigen-solver (Sec. 2, Eqs. 2-10)
-// spread over one thread-block cluster.
+// spread over one thread-block cluster, for the matrices (129 to 256 bands)
+// that take longer on one SM; and the choice between it and k_jacobi_sm.cu.
 //
 // The paper zeroes one element per host round trip (Sec. 4.2 stage 4) and
 // notes that rotations on disjoint row/column pairs commute (Sec. 2, last
@@ -55,8 +56,7 @@
 #include <algorithm>
 #include <type_traits>
 
-#include "common.cuh"
-#include "tma.cuh"
+#include "jacobi.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -77,7 +77,7 @@ constexpr int kSlots = 4;
 constexpr int kRecs = 128;        // records per slot: 32 lanes x W/2 pairs, W <= 8
 constexpr uint32_t kNone = 0xffffffffu;
 
-struct Params {
+struct alignas(kJacobiParamsBytes) Params {
   const double* C;
   int B;
   float tol32;
@@ -90,32 +90,12 @@ struct Params {
   DevHeader* hdr;
 };
 
-__device__ __forceinline__ float rcp_nr(float x) {
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return fmaf(r, fmaf(-x, r, 1.f), r);
-}
-__device__ __forceinline__ float rsqrt_nr(float x) {
-  float y;
-  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return fmaf(y, fmaf(-0.5f * x * y, y, 0.5f), y);
-}
-__device__ __forceinline__ float sqrt_est(float x) {
-  float y;
-  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-
-// Eqs. 2-5: small root t of Eq. 3 as t = sgn(tau)/(|tau| + sqrt(1+tau^2)),
-// tau = (aqq - app)/(2 apq); an off-diagonal below 2^-24 sqrt(|app aqq|) is
-// dropped without rotating (c = 1, s = 0).  Returns the record of the pair:
-// (c, s) and the two diagonal values after the rotation and position swap.
-// With d = aqq - app and n = 2 apq the same root is
-// t = sgn(tau) |n| / (|d| + sqrt(d^2 + n^2)) (sgn 0 = +1): three dependent
-// reciprocal/root steps instead of four (the step's critical path runs
-// through this record).  Where d^2 + n^2 could leave the FP32 range (|d| or
-// |n| beyond 1e18, or both below 1e-18) the scale-free tau form is taken.
-__device__ __forceinline__ float4 pair_record(float app, float aqq, float apq) {
+// pair_record (jacobi.cuh) with the drop test before the root.  The same values;
+// which one is faster depends on how the rest of the step is compiled: with
+// 224 bands 0.825 us a step with the test first, 0.811 beside
+// (188 bands 0.82 / 0.80), with 256 bands 0.905 / 0.918 -- so the test goes first
+// above 224 bands only.
+__device__ __forceinline__ float4 pair_record_drop_first(float app, float aqq, float apq) {
   const float thr = 5.9604645e-08f * sqrt_est(fabsf(app)) * sqrt_est(fabsf(aqq));
   if (!(fabsf(apq) > thr)) return make_float4(1.f, 0.f, aqq, app);
   {
@@ -143,17 +123,6 @@ __device__ __forceinline__ float4 pair_record(float app, float aqq, float apq) {
   return make_float4(c, tt * c, fmaf(tt, apq, aqq), fmaf(-tt, apq, app));
 }
 
-// M' = G_I M G_J, G = [[s, c], [c, -s]].
-__device__ __forceinline__ void rot_block(float2 csI, float2 csJ, float& m00, float& m01,
-                                          float& m10, float& m11) {
-  const float cI = csI.x, sI = csI.y, cJ = csJ.x, sJ = csJ.y;
-  const float t00 = fmaf(m00, sJ, m01 * cJ), t01 = fmaf(m00, cJ, -m01 * sJ);
-  const float t10 = fmaf(m10, sJ, m11 * cJ), t11 = fmaf(m10, cJ, -m11 * sJ);
-  m00 = fmaf(sI, t00, cI * t10);
-  m01 = fmaf(sI, t01, cI * t11);
-  m10 = fmaf(cI, t00, -sI * t10);
-  m11 = fmaf(cI, t01, -sI * t11);
-}
 
 struct Shared {
   uint64_t mbar[kSlots];  // step s+1 completes on mbar[(s + 1) % kSlots]
@@ -197,12 +166,6 @@ __device__ __forceinline__ void push_record(cg::cluster_group& cl, Shared* sh, i
   }
 }
 
-// Shared-memory address a (this CTA's window) in the window of CTA `rank`.
-__device__ __forceinline__ uint32_t mapa(uint32_t a, int rank) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
-  return r;
-}
 // Stores into a CTA of the cluster that complete-tx their bytes on that
 // CTA's mbarrier `bar` (both addresses in the receiver's window).
 __device__ __forceinline__ void st_async(uint32_t a, float x, float y, uint32_t bar) {
@@ -232,17 +195,6 @@ __device__ __forceinline__ float4 rec4(const Shared* sh, int slot, int J) {
   const int i = rix<H>(J);
   const float2 a = sh->cs[slot][i], b = sh->dd[slot][i];
   return make_float4(a.x, a.y, b.x, b.y);
-}
-// Phase wait with cluster-scope acquire (the st.async data of other CTAs).
-__device__ __forceinline__ bool mbar_try_cluster(uint64_t* b, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
-      " selp.u32 %0, 1, 0, p;\n}\n"
-      : "=r"(ok)
-      : "r"(su32(b)), "r"(parity)
-      : "memory");
-  return ok != 0;
 }
 static __device__ __noinline__ void mbar_wait_cluster_slow(uint64_t* b, uint32_t parity, int* abort) {
   const unsigned long long t0 = gtimer();
@@ -277,10 +229,13 @@ __device__ __forceinline__ const Params& par(const Params& one, const Params* li
 
 // One matrix per cluster: `one` when list is null, else list[cluster index]
 // (every entry of a list has the cluster size one.nA).
-template <int W, int VR, int MI>
+template <int W, int VR, int MI, bool kDropFirst>
 __global__ void __launch_bounds__(kThreads, 1)
 k_jacobi_cluster(const __grid_constant__ Params one, const Params* __restrict__ list) {
   constexpr int H = W / 2;                 // pairs per lane in a V row
+  auto record = [](float app, float aqq, float apq) {
+    return kDropFirst ? pair_record_drop_first(app, aqq, apq) : pair_record(app, aqq, apq);
+  };
   extern __shared__ __align__(16) float rows[];
   __shared__ Shared sh;
   cg::cluster_group cl = cg::this_cluster();
@@ -517,7 +472,7 @@ k_jacobi_cluster(const __grid_constant__ Params one, const Params* __restrict__ 
     if (tid < I_hi - I_lo) {
       const int I = I_lo + tid, p = 2 * I;
       float* apq = rows + (p - R0) * Bp + p + 1;
-      push_record<H>(cl, &sh, ncl, gs % kSlots, I, pair_record(sh.dg[p], sh.dg[p + 1], *apq));
+      push_record<H>(cl, &sh, ncl, gs % kSlots, I, record(sh.dg[p], sh.dg[p + 1], *apq));
       *apq = 0.f;
       if (I == I_lo && has_prev) cl.map_shared_rank(rows, rank - 1)[(size_t)halo_row * Bp + p + 1] = 0.f;
     }
@@ -553,7 +508,7 @@ k_jacobi_cluster(const __grid_constant__ Params one, const Params* __restrict__ 
           const float4 gI = rec4<H>(&sh, cur, I), gJ = rec4<H>(&sh, cur, I + 1);
           rot_block(make_float2(gI.x, gI.y), make_float2(gJ.x, gJ.y), m00, m01, m10, m11);
           if (!last) {  // (q_I, p_{I+1}) is the off-diagonal of a next-step pair
-            push_record_async<H>(&sh, ncl, nxt, e == 0 ? I : I + 1, pair_record(gI.w, gJ.z, m10));
+            push_record_async<H>(&sh, ncl, nxt, e == 0 ? I : I + 1, record(gI.w, gJ.z, m10));
             m10 = 0.f;
           }
           if (e == 0) {
@@ -579,7 +534,7 @@ k_jacobi_cluster(const __grid_constant__ Params one, const Params* __restrict__ 
             float n0 = fmaf(x, g.y, y * g.x);
             const float n1 = fmaf(x, g.x, -y * g.y);
             if (!last) {
-              push_record_async<H>(&sh, ncl, nxt, 0, pair_record(sh.dd[prv][rix<H>(0)].x, g.z, n0));
+              push_record_async<H>(&sh, ncl, nxt, 0, record(sh.dd[prv][rix<H>(0)].x, g.z, n0));
               n0 = 0.f;
             }
             a[0] = n0;
@@ -593,7 +548,7 @@ k_jacobi_cluster(const __grid_constant__ Params one, const Params* __restrict__ 
             float n1 = fmaf(g.x, x, -g.y * y);
             if (!last) {
               push_record_async<H>(&sh, ncl, nxt, P - 1,
-                                   pair_record(g.w, sh.dd[prv][rix<H>(P - 1)].y, n1));
+                                   record(g.w, sh.dd[prv][rix<H>(P - 1)].y, n1));
               n1 = 0.f;
             }
             a[0] = n0;
@@ -745,16 +700,8 @@ k_jacobi_cluster(const __grid_constant__ Params one, const Params* __restrict__ 
   cl.sync();  // no CTA leaves while others may still write its shared memory
 }
 
-int v_width(int Bp) { return Bp <= 64 ? 2 : (Bp <= 128 ? 4 : 8); }
 
 }  // namespace
-
-bool jacobi_cluster_shape(int B, int* nA, int* nV) {
-  const int Bp = round_even(B);
-  *nA = Bp <= 32 ? 1 : (Bp <= 64 ? 2 : (Bp <= 128 ? 4 : 8));
-  *nV = 0;
-  return true;
-}
 
 namespace {
 
@@ -768,9 +715,7 @@ size_t make_params(const double* C, int B, float tol32, int sweeps_max, bool rel
   prm.tol32 = tol32;
   prm.sweeps_max = sweeps_max;
   prm.relative_stop = relative_stop ? 1 : 0;
-  int nV = 0;
-  jacobi_cluster_shape(B, &prm.nA, &nV);
-  if (nA > 0) prm.nA = nA;
+  prm.nA = nA > 0 ? nA : kMaxCl;
   if (prm.nA > P) prm.nA = P;
   // rows: balance the blocks (I, J >= I) of the even steps
   const long total = (long)P * (P + 1) / 2;
@@ -799,18 +744,50 @@ size_t make_params(const double* C, int B, float tol32, int sweeps_max, bool rel
   return (size_t)maxrows * Bp * sizeof(float);
 }
 
+// Fewest CTAs that hold the rows of V in registers: kVRows rows per bulk warp.
+int min_ctas(int B) {
+  const int Bp = round_even(B), per = kVRows * kBulkWarps;
+  const int n = (Bp + per - 1) / per;
+  return n < 1 ? 1 : (n > kMaxCl ? kMaxCl : n);
+}
+
+// Fewest CTAs, at least n0, whose kernel variant holds the matrix: every CTA's
+// rows of V and bulk blocks of both parities within the variant's capacity (the
+// same counts the kernel checks).
+int fewest_ctas(int B, int n0) {
+  const int Bp = round_even(B), P = Bp / 2;
+  for (int n = n0 < 1 ? 1 : n0; n <= kMaxCl; ++n) {
+    Params prm;
+    make_params(nullptr, B, 1.f, 1, true, nullptr, nullptr, nullptr, n, &prm);
+    const bool wide = prm.nA < min_ctas(B);
+    const int vr = wide ? kWideVRows : kVRows, mi = wide ? kWideItems : kMaxItems;
+    bool fits = P <= 32 * 4;
+    for (int r = 0; r < prm.nA && fits; ++r) {
+      const int V0 = (int)((long)Bp * r / prm.nA), V1 = (int)((long)Bp * (r + 1) / prm.nA);
+      if (V1 - V0 > vr * kBulkWarps) fits = false;
+      for (int e = 0; e < 2 && fits; ++e) {
+        const int np = P - e, hi = std::min(prm.rp[r + 1], np - 2);
+        long total = 0;
+        for (int I = prm.rp[r]; I < hi; ++I) total += np - 2 - I;
+        if (total > (long)mi * kBulkLanes) fits = false;
+      }
+    }
+    if (fits) return prm.nA;
+  }
+  return min_ctas(B);
+}
+
 // Kernel variant: the default holds kVRows rows of V per bulk warp; clusters
 // with fewer CTAs than that needs (the batched form's throughput shapes) hold
 // kWideVRows rows and up to kWideItems bulk blocks per lane.
-cudaError_t launch_clusters(int w, const Params& one, const Params* list, int count, size_t smem,
+cudaError_t launch_clusters(const Params& one, const Params* list, int count, size_t smem,
                             cudaStream_t st) {
-  void (*kern)(const Params, const Params*);
-  const bool wide = one.nA < jacobi_min_ctas(one.B);
-  switch (w) {
-    case 2: kern = wide ? k_jacobi_cluster<2, kWideVRows, kWideItems> : k_jacobi_cluster<2, kVRows, kMaxItems>; break;
-    case 4: kern = wide ? k_jacobi_cluster<4, kWideVRows, kWideItems> : k_jacobi_cluster<4, kVRows, kMaxItems>; break;
-    default: kern = wide ? k_jacobi_cluster<8, kWideVRows, kWideItems> : k_jacobi_cluster<8, kVRows, kMaxItems>; break;
-  }
+  const bool wide = one.nA < min_ctas(one.B);
+  const bool drop_first = round_even(one.B) > 224;
+  auto kern = wide ? (drop_first ? k_jacobi_cluster<8, kWideVRows, kWideItems, true>
+                                 : k_jacobi_cluster<8, kWideVRows, kWideItems, false>)
+                   : (drop_first ? k_jacobi_cluster<8, kVRows, kMaxItems, true>
+                                 : k_jacobi_cluster<8, kVRows, kMaxItems, false>);
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
@@ -832,67 +809,63 @@ cudaError_t launch_clusters(int w, const Params& one, const Params* list, int co
 
 }  // namespace
 
+// ------------------------------------------------ which kernel a matrix takes
+// Up to 128 bands k_jacobi_sm.cu, whose matrix stays in one SM; above, the one
+// of this file: its blocks are spread over up to 8 SMs, and one SM's shared memory
+// would take longer for them than the exchange between SMs does (128 bands: 0.70
+// us a step on one SM, 0.73 here; 160 bands: 1.0 against 0.80).
+
+int jacobi_width(int B) {
+  const int Bp = round_even(B);
+  return Bp <= 64 ? 2 : (Bp <= 128 ? 4 : 8);
+}
+
+// The latency-oriented shape of the single-matrix form.
+bool jacobi_cluster_shape(int B, int* nA, int* nV) {
+  const int Bp = round_even(B);
+  const bool sm = jacobi_sm_supported(B);
+  *nA = sm ? 1 : kMaxCl;
+  *nV = sm ? (Bp <= 64 ? 1 : 3) : 0;
+  return true;
+}
+
 cudaError_t launch_jacobi_cluster(const double* C, int B, float tol32, int sweeps_max,
                                   bool relative_stop, float* diag32, float* v32, DevHeader* hdr,
                                   cudaStream_t st) {
-  Params prm;
-  const size_t smem =
-      make_params(C, B, tol32, sweeps_max, relative_stop, diag32, v32, hdr, 0, &prm);
-  return launch_clusters(v_width(round_even(B)), prm, nullptr, 1, smem, st);
+  alignas(kJacobiParamsBytes) unsigned char prm[kJacobiParamsBytes];
+  const size_t smem = jacobi_fill_params(prm, C, B, tol32, sweeps_max, relative_stop, diag32, v32, hdr, 0);
+  return launch_jacobi_cluster_list(prm, nullptr, 1, smem, st);
 }
 
-int jacobi_width(int B) { return v_width(round_even(B)); }
-
-// Fewest CTAs whose kernel variant holds the matrix: every CTA's rows of V
-// and bulk blocks of both parities within the variant's capacity (the same
-// counts the kernel checks).
-int jacobi_batch_ctas(int B) { return jacobi_ctas_at_least(B, 1); }
-
-int jacobi_ctas_at_least(int B, int n0) {
-  const int Bp = round_even(B), P = Bp / 2;
-  for (int n = n0 < 1 ? 1 : n0; n <= kMaxCl; ++n) {
-    Params prm;
-    make_params(nullptr, B, 1.f, 1, true, nullptr, nullptr, nullptr, n, &prm);
-    const bool wide = prm.nA < jacobi_min_ctas(B);
-    const int vr = wide ? kWideVRows : kVRows, mi = wide ? kWideItems : kMaxItems;
-    bool fits = P <= 32 * (v_width(Bp) / 2);
-    for (int r = 0; r < prm.nA && fits; ++r) {
-      const int V0 = (int)((long)Bp * r / prm.nA), V1 = (int)((long)Bp * (r + 1) / prm.nA);
-      if (V1 - V0 > vr * kBulkWarps) fits = false;
-      for (int e = 0; e < 2 && fits; ++e) {
-        const int np = P - e, hi = std::min(prm.rp[r + 1], np - 2);
-        long total = 0;
-        for (int I = prm.rp[r]; I < hi; ++I) total += np - 2 - I;
-        if (total > (long)mi * kBulkLanes) fits = false;
-      }
-    }
-    if (fits) return prm.nA;
-  }
-  return jacobi_min_ctas(B);
+int jacobi_ctas_at_least(int B, int n) {
+  if (!jacobi_sm_supported(B)) return fewest_ctas(B, n);
+  return std::min(kMaxCl, std::max(n, jacobi_sm_fewest(B)));
 }
 
-// Fewest CTAs that hold the rows of V in registers: kVRows rows per bulk warp.
-int jacobi_min_ctas(int B) {
-  const int Bp = round_even(B), per = kVRows * kBulkWarps;
-  const int n = (Bp + per - 1) / per;
-  return n < 1 ? 1 : (n > kMaxCl ? kMaxCl : n);
-}
-
-size_t jacobi_params_bytes() { return sizeof(Params); }
+size_t jacobi_params_bytes() { return kJacobiParamsBytes; }
 
 size_t jacobi_fill_params(void* dst, const double* C, int B, float tol32, int sweeps_max,
-                          bool relative_stop, float* diag32, float* v32, DevHeader* hdr, int nA) {
-  return make_params(C, B, tol32, sweeps_max, relative_stop, diag32, v32, hdr, nA,
-                     static_cast<Params*>(dst));
+                          bool relative_stop, float* diag32, float* v32, DevHeader* hdr, int n) {
+  if (n == 0) {
+    int nA, nV;
+    jacobi_cluster_shape(B, &nA, &nV);
+    n = nA + nV;
+  }
+  return jacobi_sm_supported(B)
+             ? jacobi_sm_fill(dst, C, B, tol32, sweeps_max, relative_stop, diag32, v32, hdr, n)
+             : make_params(C, B, tol32, sweeps_max, relative_stop, diag32, v32, hdr, n,
+                           static_cast<Params*>(dst));
 }
 
-int jacobi_params_ctas(const void* params) { return static_cast<const Params*>(params)->nA; }
-
+// dev_list null: one cluster with the host parameters.
 cudaError_t launch_jacobi_cluster_list(const void* host_first, const void* dev_list, int count,
                                        size_t smem, cudaStream_t st) {
   if (count <= 0) return cudaSuccess;
-  const Params& one = *static_cast<const Params*>(host_first);
-  return launch_clusters(v_width(round_even(one.B)), one, static_cast<const Params*>(dev_list),
+  // both parameter types begin with the matrix and its bands
+  struct Head { const double* C; int B; };
+  if (jacobi_sm_supported(static_cast<const Head*>(host_first)->B))
+    return launch_jacobi_sm(host_first, dev_list, count, smem, st);
+  return launch_clusters(*static_cast<const Params*>(host_first), static_cast<const Params*>(dev_list),
                          count, smem, st);
 }
 
