@@ -146,14 +146,14 @@ __device__ __forceinline__ PItem proj_item(const ProjArgs& one, const CUtensorMa
   return it;
 }
 
-// maxB, maxk: the largest bands and components of the items (shared-memory
-// sizing); the single-cube form takes its cube as `one` with map `tmap`.
+// maxB: the largest bands of the items (shared-memory sizing); the single-cube
+// form takes its cube as `one` with map `tmap`.
 template <typename In, int KQ, bool kTiled>
 __global__ void __launch_bounds__(kThreadsP, 1)
 k_project(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ ProjArgs one,
           const TileDesc* __restrict__ T, const CUtensorMap* __restrict__ maps,
           const ProjItem* __restrict__ items, const int* __restrict__ cta_items, int maxB,
-          int maxk, int S, int stage_bytes) {
+          int red_pad, int sync_off, int S, int stage_bytes) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   // 1024-byte aligned start (the 128-byte swizzle repeats every 1024 bytes);
   // offsetting the array itself keeps every access a shared-memory one
@@ -163,8 +163,11 @@ k_project(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ Proj
   unsigned char* stages = smem;
   float4* vs = reinterpret_cast<float4*>(stages + (size_t)S * stage_bytes);  // [B8][KQ]
   float* mus = reinterpret_cast<float*>(vs + (size_t)B8m * KQ);              // [B8]
-  float* red = mus + B8m;                                                    // [kParts][kPc][k]
-  ProjSync* sy = reinterpret_cast<ProjSync*>(red + (size_t)kParts * kPc * maxk);
+  // partial sums [kParts][kPc][kp]: kp = k, or k + 1 for even k where that fits, so
+  // that the 32 pixels of a store lie in different banks (k = 16 and 8 words apart
+  // they fell on 2 and 4; 1024 x 1024 x 200 FP16, k = 16: 488 us, 294 so)
+  float* red = mus + B8m;
+  ProjSync* sy = reinterpret_cast<ProjSync*>(reinterpret_cast<unsigned char*>(smem) + sync_off);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int nitems = T == nullptr ? 1 : cta_items[blockIdx.x + 1] - cta_items[blockIdx.x];
@@ -319,7 +322,8 @@ k_project(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ Proj
       }
     }
     // partial sums of this band part -> shared, then the eight parts are added
-    float* rp = red + (size_t)h * kPc * k;
+    const int kp = k | red_pad;
+    float* rp = red + (size_t)h * kPc * kp;
 #pragma unroll
     for (int q = 0; q < KQ; ++q) {
       const float v0[4] = {a0[q].x, a0[q].y, a0[q].z, a0[q].w};
@@ -327,17 +331,18 @@ k_project(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ Proj
 #pragma unroll
       for (int t = 0; t < 4; ++t) {
         const int j = 4 * q + t;
-        if (j < k) { rp[pa * k + j] = v0[t]; rp[pb * k + j] = v1[t]; }
+        if (j < k) { rp[pa * kp + j] = v0[t]; rp[pb * kp + j] = v1[t]; }
       }
     }
     named_sync();
     float* out = a.proj + p0 * a.q_ld;
     for (int o = tid; o < cp * k; o += kCompute) {
+      const int row = o / k, col = o - row * k;
+      const float* r0 = red + row * kp + col;
       float sum = 0.f;
 #pragma unroll
-      for (int hh = 0; hh < kParts; ++hh) sum += red[(size_t)hh * kPc * k + o];
-      const int row = o / k;
-      out[(size_t)row * a.q_ld + (o - row * k)] = sum;
+      for (int hh = 0; hh < kParts; ++hh) sum += r0[(size_t)hh * kPc * kp];
+      out[(size_t)row * a.q_ld + col] = sum;
     }
     named_sync();
   }
@@ -408,18 +413,24 @@ cudaError_t project_launch(bool tiled, const CUtensorMap& tmap, const ProjArgs& 
   const int nbox = (maxB * (int)sizeof(In) + 127) / 128;
   const int stage_bytes = tiled ? nbox * kPc * 128
                                 : (int)((((size_t)kPc * maxB * sizeof(In)) + 1023) & ~(size_t)1023);
-  const size_t fixed = (size_t)B8 * KQ * 16 + (size_t)B8 * 4 + (size_t)kParts * kPc * maxk * 4 +
-                       sizeof(ProjSync) + 1024;
   const size_t budget = 227 * 1024;
-  int stages = (int)((budget - fixed) / stage_bytes);
-  stages = stages > kMaxStages ? kMaxStages : stages;
+  auto fixed = [&](int pad) {   // V_k, mu and the partial sums
+    return ((size_t)B8 * KQ * 16 + (size_t)B8 * 4 + (size_t)kParts * kPc * (maxk | pad) * 4 + 7) & ~(size_t)7;
+  };
+  auto fit = [&](int pad) {
+    const int n = (int)((budget - fixed(pad) - sizeof(ProjSync) - 1024) / stage_bytes);
+    return n > kMaxStages ? kMaxStages : n;
+  };
+  const int pad = fit(1) >= 2 ? 1 : 0;   // 256 FP32 bands and 32 columns: no room
+  const int stages = fit(pad);
   if (stages < 2) return cudaErrorInvalidValue;
-  const size_t smem = fixed + (size_t)stages * stage_bytes;
+  const size_t sync_off = (size_t)stages * stage_bytes + fixed(pad);
+  const size_t smem = sync_off + sizeof(ProjSync) + 1024;
   auto kern = tiled ? k_project<In, KQ, true> : k_project<In, KQ, false>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  kern<<<ctas, kThreadsP, smem, st>>>(tmap, one, T, maps, items, cta_items, maxB, maxk, stages,
-                                      stage_bytes);
+  kern<<<ctas, kThreadsP, smem, st>>>(tmap, one, T, maps, items, cta_items, maxB, pad, (int)sync_off,
+                                      stages, stage_bytes);
   return cudaGetLastError();
 }
 
