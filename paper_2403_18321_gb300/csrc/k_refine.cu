@@ -72,8 +72,10 @@ __device__ __forceinline__ void dfgemm_tile(const float2* __restrict__ A,
                                             const float2* __restrict__ Bm,
                                             const float2* __restrict__ X, float2* __restrict__ D,
                                             int n, int r0, int c0) {
-  __shared__ float2 as[4][kT][kT + 1];  // as[group][k][row]
-  __shared__ float2 bs[4][kT][kT + 1];  // bs[group][k][col]
+  // as[group][k][row], bs[group][k][col]; rows of a whole number of 16-byte units,
+  // so that a thread's two values are one load
+  __shared__ __align__(16) float2 as[4][kT][kT + 2];
+  __shared__ __align__(16) float2 bs[4][kT][kT + 2];
   __shared__ float2 red[3][kT * kT];
   const int grp = threadIdx.x / kTh, t = threadIdx.x % kTh;
   const int tx = t & 7, ty = t >> 3;
@@ -118,8 +120,10 @@ __device__ __forceinline__ void dfgemm_tile(const float2* __restrict__ A,
     if (ch < nchunks) {
 #pragma unroll 4
       for (int kk = 0; kk < kT; ++kk) {
-        const float2 a0 = as[grp][kk][2 * ty], a1 = as[grp][kk][2 * ty + 1];
-        const float2 b0 = bs[grp][kk][2 * tx], b1 = bs[grp][kk][2 * tx + 1];
+        const float4 a = *reinterpret_cast<const float4*>(&as[grp][kk][2 * ty]);
+        const float4 b = *reinterpret_cast<const float4*>(&bs[grp][kk][2 * tx]);
+        const float2 a0 = make_float2(a.x, a.y), a1 = make_float2(a.z, a.w);
+        const float2 b0 = make_float2(b.x, b.y), b1 = make_float2(b.z, b.w);
         df_mac(acc[0][0], a0, b0);
         df_mac(acc[0][1], a0, b1);
         df_mac(acc[1][0], a1, b0);
