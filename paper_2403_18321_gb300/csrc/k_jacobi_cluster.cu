@@ -94,7 +94,8 @@ struct alignas(kJacobiParamsBytes) Params {
 // which one is faster depends on how the rest of the step is compiled: with
 // 224 bands 0.825 us a step with the test first, 0.811 beside
 // (188 bands 0.82 / 0.80), with 256 bands 0.905 / 0.918 -- so the test goes first
-// above 224 bands only.
+// above 224 bands, and in the wide variant (the Jacobi stage of the 256-tile
+// batch 7.5 ms, 8.5 with the test beside).
 __device__ __forceinline__ float4 pair_record_drop_first(float app, float aqq, float apq) {
   const float thr = 5.9604645e-08f * sqrt_est(fabsf(app)) * sqrt_est(fabsf(aqq));
   if (!(fabsf(apq) > thr)) return make_float4(1.f, 0.f, aqq, app);
@@ -783,11 +784,9 @@ int fewest_ctas(int B, int n0) {
 cudaError_t launch_clusters(const Params& one, const Params* list, int count, size_t smem,
                             cudaStream_t st) {
   const bool wide = one.nA < min_ctas(one.B);
-  const bool drop_first = round_even(one.B) > 224;
-  auto kern = wide ? (drop_first ? k_jacobi_cluster<8, kWideVRows, kWideItems, true>
-                                 : k_jacobi_cluster<8, kWideVRows, kWideItems, false>)
-                   : (drop_first ? k_jacobi_cluster<8, kVRows, kMaxItems, true>
-                                 : k_jacobi_cluster<8, kVRows, kMaxItems, false>);
+  auto kern = wide ? k_jacobi_cluster<8, kWideVRows, kWideItems, true>
+              : round_even(one.B) > 224 ? k_jacobi_cluster<8, kVRows, kMaxItems, true>
+                                        : k_jacobi_cluster<8, kVRows, kMaxItems, false>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
