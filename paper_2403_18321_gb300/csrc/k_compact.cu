@@ -38,6 +38,7 @@ __device__ __forceinline__ void compact_row(int i, const float* __restrict__ dia
 __global__ void k_compact(const float* __restrict__ diag32, const float* __restrict__ v32, int B,
                           DevHeader* __restrict__ hdr, double* __restrict__ lam,
                           float2* __restrict__ vc) {
+  pdl_begin();
   compact_row(blockIdx.x, diag32, v32, B, hdr, lam, vc);
 }
 __global__ void k_compact_batched(const TileDesc* __restrict__ T) {
@@ -50,8 +51,7 @@ __global__ void k_compact_batched(const TileDesc* __restrict__ T) {
 
 cudaError_t launch_compact(const float* diag32, const float* v32, int B, DevHeader* hdr,
                            double* lam, float2* vc, cudaStream_t st) {
-  k_compact<<<B, 256, 0, st>>>(diag32, v32, B, hdr, lam, vc);
-  return cudaGetLastError();
+  return launch_after(k_compact, B, 256, 0, st, diag32, v32, B, hdr, lam, vc);
 }
 
 cudaError_t launch_compact_batched(const TileDesc* T, int ntiles, int maxB, cudaStream_t st) {

@@ -215,6 +215,7 @@ k_syrk_simt(const In* __restrict__ cube, int64_t N, int B, int parts, float* __r
             const int* __restrict__ guard, int* __restrict__ escale) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   if constexpr (kGuarded) {
+    pdl_begin();
     if (*(volatile const int*)guard == 0) return;
     for (int g = blockIdx.x; g < parts; g += gridDim.x) {
       syrk_simt_cta<In, Acc, TM>(cube, B, N * g / parts, N * (g + 1) / parts, g, blockIdx.y,
@@ -287,6 +288,9 @@ cudaError_t syrk_simt_typed(const In* cube, int64_t N, int B, bool fp64, float* 
                         16 + kAhead * sizeof(float4) * (size_t)raw_units(Bt * TM, (int)sizeof(In));
     auto kern = guard != nullptr ? k_syrk_simt<In, double, TM, true> : k_syrk_simt<In, double, TM, false>;
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (guard != nullptr)
+      return launch_after(kern, dim3(gx, groups), threads, smem, st, cube, N, B, partials, shift, s1_part,
+                          (double*)s2_part, guard, escale);
     kern<<<dim3(gx, groups), threads, smem, st>>>(cube, N, B, partials, shift, s1_part,
                                                        (double*)s2_part, guard, escale);
   } else {
@@ -298,6 +302,9 @@ cudaError_t syrk_simt_typed(const In* cube, int64_t N, int B, bool fp64, float* 
                         16 + kAhead * sizeof(float4) * (size_t)raw_units(Bt * TM, (int)sizeof(In));
     auto kern = guard != nullptr ? k_syrk_simt<In, float, TM, true> : k_syrk_simt<In, float, TM, false>;
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (guard != nullptr)
+      return launch_after(kern, dim3(gx, groups), threads, smem, st, cube, N, B, partials, shift, s1_part,
+                          (float*)s2_part, guard, escale);
     kern<<<dim3(gx, groups), threads, smem, st>>>(cube, N, B, partials, shift, s1_part,
                                                        (float*)s2_part, guard, escale);
   }
@@ -361,6 +368,7 @@ __global__ void k_s1_reduce(const double* __restrict__ s1_part, int partials, in
                             const float* __restrict__ shift, double* __restrict__ dvec,
                             double* __restrict__ mu, float* __restrict__ mu_f,
                             DevHeader* __restrict__ hdr) {
+  pdl_begin();
   s1_reduce_band(blockIdx.x, s1_part, partials, B, N, shift, dvec, mu, mu_f, hdr);
 }
 __global__ void k_s1_reduce_batched(const TileDesc* __restrict__ T) {
@@ -439,6 +447,7 @@ __global__ void __launch_bounds__(kFinWarps * 32)
 k_cov_finalize(const Acc* __restrict__ s2_part, int partials, int s2_elems, int B, int64_t N,
                const double* __restrict__ dvec, double* __restrict__ C,
                DevHeader* __restrict__ hdr, const int* __restrict__ escale) {
+  pdl_begin();
   cov_finalize_block<Acc>(blockIdx.x, s2_part, partials, s2_elems, B, N, dvec, C, hdr, escale);
 }
 template <typename Acc>
@@ -474,16 +483,16 @@ cudaError_t launch_cov_finalize(const float* shift, const double* s1_part, const
                                 bool fp64_partials, int partials, int64_t N, int B, double* mu,
                                 double* C, float* mu_f, double* dvec, DevHeader* hdr,
                                 cudaStream_t st, const int* escale) {
-  k_s1_reduce<<<B, 32, 0, st>>>(s1_part, partials, B, N, shift, dvec, mu, mu_f, hdr);
+  const cudaError_t e =
+      launch_after(k_s1_reduce, B, 32, 0, st, s1_part, partials, B, N, shift, dvec, mu, mu_f, hdr);
+  if (e != cudaSuccess) return e;
   const int s2_elems = B * (B + 1) / 2;
   const int grid = (s2_elems + 31) / 32;
   if (fp64_partials)
-    k_cov_finalize<double><<<grid, kFinWarps * 32, 0, st>>>((const double*)s2_part, partials,
-                                                            s2_elems, B, N, dvec, C, hdr, escale);
-  else
-    k_cov_finalize<float><<<grid, kFinWarps * 32, 0, st>>>((const float*)s2_part, partials,
-                                                           s2_elems, B, N, dvec, C, hdr, escale);
-  return cudaGetLastError();
+    return launch_after(k_cov_finalize<double>, grid, kFinWarps * 32, 0, st, (const double*)s2_part,
+                        partials, s2_elems, B, N, dvec, C, hdr, escale);
+  return launch_after(k_cov_finalize<float>, grid, kFinWarps * 32, 0, st, (const float*)s2_part,
+                      partials, s2_elems, B, N, dvec, C, hdr, escale);
 }
 
 cudaError_t launch_syrk_simt_grouped(const TileDesc* T, const CovItem* items, int nitems,

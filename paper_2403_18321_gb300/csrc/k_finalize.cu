@@ -58,6 +58,7 @@ __device__ __forceinline__ void rank_sign_pair(int j, const double* __restrict__
 __global__ void __launch_bounds__(256)
 k_rank_sign(const double* __restrict__ lam, const float2* __restrict__ vc, int B,
             int* __restrict__ rank, double* __restrict__ sgn, double* __restrict__ eigvals) {
+  pdl_begin();
   rank_sign_pair(blockIdx.x, lam, vc, B, rank, sgn, eigvals);
 }
 
@@ -77,6 +78,7 @@ __device__ __forceinline__ void scatter_row(int i, const float2* __restrict__ vc
 __global__ void __launch_bounds__(256)
 k_scatter(const float2* __restrict__ vc, int B, int k, const int* __restrict__ rank,
           const double* __restrict__ sgn, double* __restrict__ eigvecs, float* __restrict__ vk) {
+  pdl_begin();
   scatter_row(blockIdx.x, vc, B, k, rank, sgn, eigvecs, vk);
 }
 __global__ void __launch_bounds__(256)
@@ -93,6 +95,7 @@ k_scatter_batched(const TileDesc* __restrict__ T, int in_w) {
 }
 __global__ void k_narrow(const double* __restrict__ mu, const double* __restrict__ V, int B, int k,
                          float* __restrict__ mu_f, float* __restrict__ vk) {
+  pdl_begin();
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < B * k; e += gridDim.x * blockDim.x) {
     const int i = e / k, j = e - i * k;
     vk[e] = (float)V[(size_t)i * B + j];
@@ -105,15 +108,14 @@ __global__ void k_narrow(const double* __restrict__ mu, const double* __restrict
 
 cudaError_t launch_narrow_inputs(const double* mu, const double* eigvecs, int B, int k, float* mu_f,
                                  float* vk, cudaStream_t st) {
-  k_narrow<<<(B * k + 255) / 256, 256, 0, st>>>(mu, eigvecs, B, k, mu_f, vk);
-  return cudaGetLastError();
+  return launch_after(k_narrow, (B * k + 255) / 256, 256, 0, st, mu, eigvecs, B, k, mu_f, vk);
 }
 
 cudaError_t launch_sort_sign(const double* lam, const float2* vc, int B, int k, double* eigvals,
                              double* eigvecs, float* vk, int* rank, double* sgn, cudaStream_t st) {
-  k_rank_sign<<<B, 256, 0, st>>>(lam, vc, B, rank, sgn, eigvals);
-  k_scatter<<<B, 256, 0, st>>>(vc, B, k, rank, sgn, eigvecs, vk);
-  return cudaGetLastError();
+  const cudaError_t e = launch_after(k_rank_sign, B, 256, 0, st, lam, vc, B, rank, sgn, eigvals);
+  if (e != cudaSuccess) return e;
+  return launch_after(k_scatter, B, 256, 0, st, vc, B, k, rank, sgn, eigvecs, vk);
 }
 
 cudaError_t launch_sort_sign_batched(const TileDesc* T, int ntiles, int maxB, bool final_in_w,

@@ -170,6 +170,7 @@ k_project(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ Proj
   ProjSync* sy = reinterpret_cast<ProjSync*>(reinterpret_cast<unsigned char*>(smem) + sync_off);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  pdl_wait();
   const int nitems = T == nullptr ? 1 : cta_items[blockIdx.x + 1] - cta_items[blockIdx.x];
   if (T == nullptr && one.guard != nullptr && *(volatile const int*)one.guard == 0) return;
 
@@ -429,9 +430,8 @@ cudaError_t project_launch(bool tiled, const CUtensorMap& tmap, const ProjArgs& 
   auto kern = tiled ? k_project<In, KQ, true> : k_project<In, KQ, false>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  kern<<<ctas, kThreadsP, smem, st>>>(tmap, one, T, maps, items, cta_items, maxB, pad, (int)sync_off,
-                                      stages, stage_bytes);
-  return cudaGetLastError();
+  return launch_after(kern, ctas, kThreadsP, smem, st, tmap, one, T, maps, items, cta_items, maxB, pad,
+                      (int)sync_off, stages, stage_bytes);
 }
 
 template <typename In>

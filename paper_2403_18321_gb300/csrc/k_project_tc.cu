@@ -98,6 +98,7 @@ template <typename In>
 __global__ void __launch_bounds__(256)
 k_ptc_bands(const In* __restrict__ cube, int64_t N, int B, const double* __restrict__ mu,
             float* __restrict__ shift, int* __restrict__ escale) {
+  pdl_begin();
   const int b = threadIdx.x;
   if (b >= B) return;
   const float s = on_grid<In>((float)mu[b]);
@@ -134,6 +135,7 @@ k_ptc_vop(const double* __restrict__ V, int B, int j0, int k, const double* __re
           const float* __restrict__ shift, const int* __restrict__ escale,
           unsigned char* __restrict__ planes, float* __restrict__ colscale,
           float* __restrict__ corr) {
+  pdl_begin();
   __shared__ float wmax[8];
   __shared__ double csum[8];
   const int j = blockIdx.x, b = threadIdx.x, lane = b & 31, warp = b >> 5;
@@ -690,14 +692,13 @@ cudaError_t launch_project_tc(const void* cube, pca_dtype dt, int64_t N, int B, 
   if (N < 1) return cudaSuccess;
   switch (dt) {
     case PCA_F32:
-      k_ptc_bands<float><<<1, 256, 0, st>>>((const float*)cube, N, B, mu, shift, escale);
+      launch_after(k_ptc_bands<float>, 1, 256, 0, st, (const float*)cube, N, B, mu, shift, escale);
       break;
     case PCA_BF16:
-      k_ptc_bands<__nv_bfloat16><<<1, 256, 0, st>>>((const __nv_bfloat16*)cube, N, B, mu, shift,
-                                                     escale);
+      launch_after(k_ptc_bands<__nv_bfloat16>, 1, 256, 0, st, (const __nv_bfloat16*)cube, N, B, mu, shift, escale);
       break;
     case PCA_F16:
-      k_ptc_bands<__half><<<1, 256, 0, st>>>((const __half*)cube, N, B, mu, shift, escale);
+      launch_after(k_ptc_bands<__half>, 1, 256, 0, st, (const __half*)cube, N, B, mu, shift, escale);
       break;
     default:
       return cudaErrorInvalidValue;
@@ -708,7 +709,7 @@ cudaError_t launch_project_tc(const void* cube, pca_dtype dt, int64_t N, int B, 
   for (int j0 = 0; j0 < k; j0 += kMaxCols) {
     const int kk = k - j0 < kMaxCols ? k - j0 : kMaxCols;
     const int N16 = (kk + 15) & ~15;
-    k_ptc_vop<<<N16, 256, 0, st>>>(V, B, j0, kk, mu, shift, escale, planes, colscale, corr);
+    launch_after(k_ptc_vop, N16, 256, 0, st, V, B, j0, kk, mu, shift, escale, planes, colscale, corr);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const PtcArgs a{cube, N, B, kk, N16, k, proj + j0, shift, escale, planes, colscale, corr, hdr};
     switch (dt) {

@@ -162,6 +162,7 @@ template <bool kTransA>
 __global__ void __launch_bounds__(kTh * 4)
 k_dfgemm(const float2* __restrict__ A, const float2* __restrict__ Bm,
          const float2* __restrict__ X, float2* __restrict__ D, int n, int sym) {
+  pdl_begin();
   if (sym && blockIdx.y > blockIdx.x) return;
   dfgemm_tile<kTransA>(A, Bm, X, D, n, blockIdx.y * kT, blockIdx.x * kT);
 }
@@ -192,8 +193,8 @@ k_dfgemm_batched(const TileDesc* __restrict__ T, int product, int flip) {
 void dfgemm(bool transA, const float2* A, const float2* Bm, const float2* X, float2* D, int n,
             bool sym, cudaStream_t st) {
   const dim3 grid((n + kT - 1) / kT, (n + kT - 1) / kT);
-  if (transA) k_dfgemm<true><<<grid, kTh * 4, 0, st>>>(A, Bm, X, D, n, sym ? 1 : 0);
-  else k_dfgemm<false><<<grid, kTh * 4, 0, st>>>(A, Bm, X, D, n, sym ? 1 : 0);
+  launch_after(transA ? k_dfgemm<true> : k_dfgemm<false>, grid, kTh * 4, 0, st, A, Bm, X, D, n,
+               sym ? 1 : 0);   // (an error stays for cudaGetLastError)
 }
 
 __device__ __forceinline__ void atomic_max_pos(double* addr, double v) {
@@ -257,6 +258,7 @@ __device__ __forceinline__ void refine_E_row(int i, int j, const float2* __restr
 }
 __global__ void k_refine_lam(const float2* __restrict__ S, const float2* __restrict__ G, int n,
                              double* __restrict__ lam, DevHeader* __restrict__ hdr) {
+  pdl_begin();
   refine_lam_entry(blockIdx.x * blockDim.x + threadIdx.x, S, G, n, lam, hdr);
 }
 __global__ void k_refine_lam_batched(const TileDesc* __restrict__ T) {
@@ -266,6 +268,7 @@ __global__ void k_refine_lam_batched(const TileDesc* __restrict__ T) {
 __global__ void k_refine_E(const float2* __restrict__ S, const float2* __restrict__ G, int n,
                            float2* __restrict__ E, const double* __restrict__ lam,
                            DevHeader* __restrict__ hdr, double inv_max_angle) {
+  pdl_begin();
   refine_E_row(blockIdx.y, blockIdx.x * blockDim.x + threadIdx.x, S, G, n, E, lam, hdr,
                inv_max_angle);
 }
@@ -286,6 +289,7 @@ __device__ __forceinline__ void ns_E_entry(int i, int j, const float2* __restric
   E[(size_t)i * n + j] = make_float2(0.5f * r.x, 0.5f * r.y);
 }
 __global__ void k_ns_E(const float2* __restrict__ G, int n, float2* __restrict__ E) {
+  pdl_begin();
   ns_E_entry(blockIdx.y, blockIdx.x * blockDim.x + threadIdx.x, G, n, E);
 }
 __global__ void k_ns_E_batched(const TileDesc* __restrict__ T) {
@@ -295,6 +299,7 @@ __global__ void k_ns_E_batched(const TileDesc* __restrict__ T) {
 }
 
 __global__ void k_to_df(const double* __restrict__ src, float2* __restrict__ dst, int count) {
+  pdl_begin();
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < count; e += gridDim.x * blockDim.x)
     dst[e] = d_to_df(src[e]);
 }
@@ -308,14 +313,13 @@ __global__ void k_to_df_batched(const TileDesc* __restrict__ T) {
 }  // namespace
 
 cudaError_t launch_to_df(const double* src, float2* dst, int count, cudaStream_t st) {
-  k_to_df<<<(count + 255) / 256, 256, 0, st>>>(src, dst, count);
-  return cudaGetLastError();
+  return launch_after(k_to_df, (count + 255) / 256, 256, 0, st, src, dst, count);
 }
 
 cudaError_t launch_orthonormalize(const float2* v, float2* vout, int B, float2* g, float2* e,
                                   cudaStream_t st) {
   dfgemm(true, v, v, nullptr, g, B, true, st);                   // G = V^T V (upper)
-  k_ns_E<<<dim3((B + 127) / 128, B), 128, 0, st>>>(g, B, e);
+  launch_after(k_ns_E, dim3((B + 127) / 128, B), 128, 0, st, g, B, e);
   dfgemm(false, v, e, v, vout, B, false, st);                    // V' = V E + V
   return cudaGetLastError();
 }
@@ -326,8 +330,8 @@ cudaError_t launch_refine(const float2* C, int B, const float2* v, float2* vout,
   dfgemm(false, C, v, nullptr, vout, B, false, st);  // W = C V (in vout until the last product)
   dfgemm(true, v, vout, nullptr, s, B, true, st);    // S = V^T W (upper)
   dfgemm(true, v, v, nullptr, g, B, true, st);       // G = V^T V (upper)
-  k_refine_lam<<<(B + 127) / 128, 128, 0, st>>>(s, g, B, lam, hdr);
-  k_refine_E<<<dim3((B + 127) / 128, B), 128, 0, st>>>(s, g, B, e, lam, hdr, 1.0 / max_angle);
+  launch_after(k_refine_lam, (B + 127) / 128, 128, 0, st, s, g, B, lam, hdr);
+  launch_after(k_refine_E, dim3((B + 127) / 128, B), 128, 0, st, s, g, B, e, lam, hdr, 1.0 / max_angle);
   dfgemm(false, v, e, v, vout, B, false, st);        // V' = V E + V
   return cudaGetLastError();
 }
