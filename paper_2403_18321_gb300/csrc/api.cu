@@ -102,9 +102,12 @@ Layout make_layout(int64_t N, int B, int k, pca_dtype dt, pca_precision prec, in
     const int64_t per_cta = (nchunk + L.tc_ctas - 1) / L.tc_ctas;
     L.partials = L.tc_ctas * (int)((per_cta + cap - 1) / cap);
     L.s2_bytes_el = 4;
+  } else if (prec == PCA_PREC_P64) {
+    L.partials = syrk_digits_parts(N, B, num_sms);
+    L.s2_bytes_el = 8;
   } else {
     L.partials = (int)std::min<int64_t>(kMaxPartials, std::max<int64_t>(1, (N + 255) / 256));
-    L.s2_bytes_el = prec == PCA_PREC_P64 ? 8 : 4;
+    L.s2_bytes_el = 4;
   }
   L.s2_elems = B * (B + 1) / 2;
   const size_t BB8 = sizeof(double) * (size_t)B * B;
@@ -113,6 +116,7 @@ Layout make_layout(int64_t N, int B, int k, pca_dtype dt, pca_precision prec, in
   L.hdr = take(sizeof(DevHeader));
   L.shift = take(sizeof(float) * B);
   L.escale = take(sizeof(int) * B);
+  L.ext = take(sizeof(unsigned) * 2 * B);
   L.s1_part = take(sizeof(double) * (size_t)L.partials * B);
   L.s2_part = take((size_t)L.s2_bytes_el * L.partials * L.s2_elems);
   L.dvec = take(sizeof(double) * B);
@@ -225,6 +229,7 @@ struct Ptrs {
   DevHeader* hdr;
   float* shift;
   int* escale;
+  unsigned* ext;
   double* s1p;
   void* s2p;
   double* dvec;
@@ -255,6 +260,7 @@ Ptrs carve(void* workspace, const Layout& L) {
   p.hdr = reinterpret_cast<DevHeader*>(ws + L.hdr);
   p.shift = reinterpret_cast<float*>(ws + L.shift);
   p.escale = reinterpret_cast<int*>(ws + L.escale);
+  p.ext = reinterpret_cast<unsigned*>(ws + L.ext);
   p.s1p = reinterpret_cast<double*>(ws + L.s1_part);
   p.s2p = ws + L.s2_part;
   p.dvec = reinterpret_cast<double*>(ws + L.dvec);
@@ -293,8 +299,13 @@ cudaError_t run_cov(const void* cube, pca_dtype dt, int64_t N, int B, pca_precis
     // (its CTAs return at once when the flag is clear)
     e = launch_syrk_simt(cube, dt, N, B, false, P.shift, P.s1p, P.s2p, L.partials, st,
                          &P.hdr->cov_range, P.escale);
+  } else if (prec == PCA_PREC_P64) {
+    e = launch_syrk_digits(cube, dt, N, B, P.shift, P.s1p, (double*)P.s2p, L.partials, P.ext, P.hdr, st);
+    if (e != cudaSuccess) return e;
+    e = launch_syrk_simt(cube, dt, N, B, true, P.shift, P.s1p, P.s2p, L.partials, st,
+                         &P.hdr->fx_range);
   } else {
-    e = launch_syrk_simt(cube, dt, N, B, prec == PCA_PREC_P64, P.shift, P.s1p, P.s2p, L.partials, st);
+    e = launch_syrk_simt(cube, dt, N, B, false, P.shift, P.s1p, P.s2p, L.partials, st);
   }
   if (e != cudaSuccess) return e;
   pm.mark(1);
@@ -635,14 +646,14 @@ int pca_version(void) { return 100; }
 
 int pca_kernel_launches(pca_precision prec, int k) {
   // header init, covariance (MIX: tensor-core pass + guarded SIMT
-  // re-computation), band-sum reduce, covariance finalise, Jacobi (with
+  // re-computation; P64: band ranges + digit products + guarded SIMT), band-sum reduce, covariance finalise, Jacobi (with
   // V), compact, 6 per refinement iteration (four products, the eigenvalue
   // and the angle kernels), 1 conversion, 3 per orthogonalisation step,
   // rank/sign + scatter, projection: one SIMT pass per 32 columns (MIX: band
   // constants, then operand preparation + tensor-core pass per 128 columns,
   // and the guarded SIMT passes)
   const int it = refine_iterations(prec);
-  const int cov = prec == PCA_PREC_MIX ? 2 : 1;
+  const int cov = prec == PCA_PREC_MIX ? 2 : prec == PCA_PREC_P64 ? 3 : 1;
   int proj = 0;
   if (k > 0) {
     proj = (k + 31) / 32;

@@ -25,6 +25,8 @@ struct DevHeader {
   int dummy_slot;    // slot of the padding index when B is odd, else -1
   int cov_range;     // tensor-core covariance met a value outside its scaled FP16 range
   int proj_range;    // tensor-core projection met a value outside its scaled FP16 range
+  int fx_range;      // a band has no fixed-point form (P64 covariance): the FP64 SIMT form runs
+  int pad;
   double off_rel;
   double fro;
   double tol_used;
@@ -34,7 +36,7 @@ struct DevHeader {
 
 // Offsets (bytes) of every workspace region; all 256-byte aligned.
 struct Layout {
-  size_t hdr, shift, escale, s1_part, s2_part, dvec, cov, cdf, rank, sgn, diag32, v32, lam, vc, w, s, r, e, vk, muf;
+  size_t hdr, shift, escale, ext, s1_part, s2_part, dvec, cov, cdf, rank, sgn, diag32, v32, lam, vc, w, s, r, e, vk, muf;
   size_t ptc_shift, ptc_escale, ptc_planes, ptc_colscale, ptc_corr;   // tensor-core projection
   size_t total;
   int partials;      // number of covariance partial slots the SYRK uses
@@ -156,6 +158,14 @@ struct ProjItem {
 cudaError_t launch_syrk_simt(const void* cube, pca_dtype dt, int64_t N, int B, bool fp64,
                              float* shift, double* s1_part, void* s2_part, int partials,
                              cudaStream_t st, const int* guard = nullptr, int* escale = nullptr);
+
+// FP64 covariance partials from exact products of 8-bit digits on the tensor cores;
+// ext: 2 B words of scratch.  A band without a fixed-point form sets hdr->fx_range, and
+// the caller's guarded SIMT launch forms the partials.
+int syrk_digits_parts(int64_t N, int B, int num_sms);   // partial slots
+cudaError_t launch_syrk_digits(const void* cube, pca_dtype dt, int64_t N, int B, float* shift,
+                               double* s1_part, double* s2_part, int parts, unsigned* ext,
+                               DevHeader* hdr, cudaStream_t st);
 
 // Covariance partials on the tensor cores (tcgen05, split-FP16 of the scaled,
 // shifted values, three products).  Every CTA derives the per-band shift
