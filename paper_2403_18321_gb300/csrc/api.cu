@@ -102,13 +102,12 @@ Layout make_layout(int64_t N, int B, int k, pca_dtype dt, pca_precision prec, in
     const int64_t per_cta = (nchunk + L.tc_ctas - 1) / L.tc_ctas;
     L.partials = L.tc_ctas * (int)((per_cta + cap - 1) / cap);
     L.s2_bytes_el = 4;
-  } else if (prec == PCA_PREC_P64) {
-    L.partials = syrk_digits_parts(N, B, num_sms);
-    L.s2_bytes_el = 8;
   } else {
     L.partials = (int)std::min<int64_t>(kMaxPartials, std::max<int64_t>(1, (N + 255) / 256));
-    L.s2_bytes_el = 4;
+    if (prec == PCA_PREC_P64) L.dig_parts = syrk_digits_parts(N, B, num_sms);
+    L.s2_bytes_el = prec == PCA_PREC_P64 ? 8 : 4;
   }
+  const size_t slots = (size_t)std::max(L.partials, L.dig_parts);
   L.s2_elems = B * (B + 1) / 2;
   const size_t BB8 = sizeof(double) * (size_t)B * B;
   size_t o = 0;
@@ -117,8 +116,8 @@ Layout make_layout(int64_t N, int B, int k, pca_dtype dt, pca_precision prec, in
   L.shift = take(sizeof(float) * B);
   L.escale = take(sizeof(int) * B);
   L.ext = take(sizeof(unsigned) * 2 * B);
-  L.s1_part = take(sizeof(double) * (size_t)L.partials * B);
-  L.s2_part = take((size_t)L.s2_bytes_el * L.partials * L.s2_elems);
+  L.s1_part = take(sizeof(double) * slots * B);
+  L.s2_part = take((size_t)L.s2_bytes_el * slots * L.s2_elems);
   L.dvec = take(sizeof(double) * B);
   L.cov = take(BB8);
   L.cdf = take(BB8);
@@ -286,10 +285,16 @@ Ptrs carve(void* workspace, const Layout& L) {
   return p;
 }
 
-// stages 2-3 of Algorithm 1: band means and covariance in one pass over the cube
+// stages 2-3 of Algorithm 1: band means and covariance in one pass over the cube.
+// digits (P64): exact products of digits on the tensor cores, the covariance call's form
+// only.  A fit keeps the FP64 sums in their order: another rounding of C, though nearer to
+// the exact one, moves the eigenvectors of close pairs (by 1e-9 where the gap is 1e-6
+// of the largest eigenvalue).
 cudaError_t run_cov(const void* cube, pca_dtype dt, int64_t N, int B, pca_precision prec,
-                    const Layout& L, const Ptrs& P, double* mu, cudaStream_t st, StageMark& pm) {
+                    const Layout& L, const Ptrs& P, double* mu, cudaStream_t st, StageMark& pm,
+                    bool digits = false) {
   cudaError_t e;
+  const int parts = digits ? L.dig_parts : L.partials;
   pm.mark(0);
   if (prec == PCA_PREC_MIX) {
     e = launch_syrk_tc(cube, dt, N, B, P.shift, P.escale, P.s1p, (float*)P.s2p, L.partials,
@@ -299,17 +304,16 @@ cudaError_t run_cov(const void* cube, pca_dtype dt, int64_t N, int B, pca_precis
     // (its CTAs return at once when the flag is clear)
     e = launch_syrk_simt(cube, dt, N, B, false, P.shift, P.s1p, P.s2p, L.partials, st,
                          &P.hdr->cov_range, P.escale);
-  } else if (prec == PCA_PREC_P64) {
-    e = launch_syrk_digits(cube, dt, N, B, P.shift, P.s1p, (double*)P.s2p, L.partials, P.ext, P.hdr, st);
+  } else if (digits) {
+    e = launch_syrk_digits(cube, dt, N, B, P.shift, P.s1p, (double*)P.s2p, parts, P.ext, P.hdr, st);
     if (e != cudaSuccess) return e;
-    e = launch_syrk_simt(cube, dt, N, B, true, P.shift, P.s1p, P.s2p, L.partials, st,
-                         &P.hdr->fx_range);
+    e = launch_syrk_simt(cube, dt, N, B, true, P.shift, P.s1p, P.s2p, parts, st, &P.hdr->fx_range);
   } else {
-    e = launch_syrk_simt(cube, dt, N, B, false, P.shift, P.s1p, P.s2p, L.partials, st);
+    e = launch_syrk_simt(cube, dt, N, B, prec == PCA_PREC_P64, P.shift, P.s1p, P.s2p, parts, st);
   }
   if (e != cudaSuccess) return e;
   pm.mark(1);
-  return launch_cov_finalize(P.shift, P.s1p, P.s2p, L.s2_bytes_el == 8, L.partials, N, B, mu, P.C,
+  return launch_cov_finalize(P.shift, P.s1p, P.s2p, L.s2_bytes_el == 8, parts, N, B, mu, P.C,
                              P.muf, P.dvec, P.hdr, st, prec == PCA_PREC_MIX ? P.escale : nullptr);
 }
 
@@ -393,7 +397,7 @@ int pca_covariance(const void* cube, pca_dtype dt, int64_t N, int B, pca_precisi
   StageMark pm(st);
   k_header_init<<<1, 1, 0, st>>>(P.hdr, 0, 0.f);
   GB_CK(cudaGetLastError());
-  GB_CK(run_cov(cube, dt, N, B, prec, L, P, mu, st, pm));
+  GB_CK(run_cov(cube, dt, N, B, prec, L, P, mu, st, pm, prec == PCA_PREC_P64));
   GB_CK(cudaMemcpyAsync(cov, P.C, sizeof(double) * (size_t)B * B, cudaMemcpyDeviceToDevice, st));
   if (info) return pca_read_info(workspace, stream, info);
   return PCA_OK;
@@ -646,14 +650,14 @@ int pca_version(void) { return 100; }
 
 int pca_kernel_launches(pca_precision prec, int k) {
   // header init, covariance (MIX: tensor-core pass + guarded SIMT
-  // re-computation; P64: band ranges + digit products + guarded SIMT), band-sum reduce, covariance finalise, Jacobi (with
+  // re-computation), band-sum reduce, covariance finalise, Jacobi (with
   // V), compact, 6 per refinement iteration (four products, the eigenvalue
   // and the angle kernels), 1 conversion, 3 per orthogonalisation step,
   // rank/sign + scatter, projection: one SIMT pass per 32 columns (MIX: band
   // constants, then operand preparation + tensor-core pass per 128 columns,
   // and the guarded SIMT passes)
   const int it = refine_iterations(prec);
-  const int cov = prec == PCA_PREC_MIX ? 2 : prec == PCA_PREC_P64 ? 3 : 1;
+  const int cov = prec == PCA_PREC_MIX ? 2 : 1;
   int proj = 0;
   if (k > 0) {
     proj = (k + 31) / 32;

@@ -40,6 +40,7 @@ struct Layout {
   size_t ptc_shift, ptc_escale, ptc_planes, ptc_colscale, ptc_corr;   // tensor-core projection
   size_t total;
   int partials;      // number of covariance partial slots the SYRK uses
+  int dig_parts;     // P64: partial slots of the covariance call's digit products
   int tc_ctas;       // MIX: CTAs of the tensor-core pass (partials spread over them)
   int s2_elems;      // packed upper-triangle entries per partial: B(B+1)/2
   int s2_bytes_el;   // 4 (FP32 partials) or 8 (FP64 partials)
