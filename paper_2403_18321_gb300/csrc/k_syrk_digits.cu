@@ -20,8 +20,9 @@
 // or a spread too small for an FP32 scale sets hdr->fx_range, and the FP64 SIMT
 // form (guarded by it) does the work.
 //
-// The covariance call, 350 x 350 x 188 FP32: 4.74 ms with the FP64 products, 1.02 ms with these.  The
-// covariance's error against extended precision, over cubes of 28,000 to 57,000 pixels and
+// The covariance call, FP64 products -> these: 350 x 350 x 188 FP32 4.74 -> 0.61 ms,
+// 610 x 340 x 103 2.88 -> 0.51, 512 x 512 x 224 BF16 13.7 -> 1.22, 10,000 x 50 0.189 -> 0.058.
+// Its error against extended precision, over cubes of 28,000 to 57,000 pixels and
 // 51 to 244 bands (relative to sqrt(C_aa C_bb), root mean square): FP64 products
 // 8e-17 .. 1.1e-15, these 9e-17 .. 1.4e-16.
 //
@@ -39,16 +40,21 @@ namespace {
 
 constexpr int kTile = 64;             // bands of a tile
 constexpr int kPx = 32;               // pixels of a chunk
-constexpr int kDigits = 7;
 constexpr int kRow = kTile + 8;       // halves of a pixel's row: eight rows fall on all banks
-constexpr int kThr = 128;             // 2 x 2 warps of 32 x 32 outputs
+constexpr int kThr = 256;             // 2 x 4 warps of 32 x 16 outputs
+
+constexpr int kDigits = 7;
 constexpr unsigned long long kBias = 0x80808080808080ull;   // digit = byte - 128
-constexpr size_t kBlockBytes = (size_t)kDigits * kPx * kRow * 2;
+constexpr int kBlockHalves = kDigits * kPx * kRow;
+constexpr size_t kBlockBytes = 2 * (size_t)kBlockHalves;
+
+// A raw row: 64 values and one more 16-byte unit, for a start between units.
+template <typename In>
+constexpr int raw_row() { return kTile * (int)sizeof(In) + 16; }
 
 struct FxSync {
   long long q0[2][kTile];    // fixed-point shift of every band of the two blocks
-  float scale[2][kTile];     // its power-of-two scale
-  int k[2][kTile];           // the exponent of the scale
+  int k[2][kTile];           // the exponent of its scale
   unsigned used[2][2];       // OR of the digits' bytes (without bias), low and high word, by chunk parity
   unsigned used_b[2][2];
   int bad;
@@ -104,8 +110,10 @@ k_band_range(const In* __restrict__ cube, int64_t N, int B, unsigned* __restrict
   }
 }
 
-// The scale 2^k of a band about its shift s: |x| 2^k < 2^54, |y| 2^k < 2^61.  False: no
-// such scale (a non-finite value, or a spread too small).
+// The scale 2^k of a band about its shift s: |x| 2^k < 2^54, and |y| 2^k < 2^61 (which only
+// bands whose values all lie within 2^-7 of each other reach: their digits then end at
+// D_2, so that nothing is left out).  False: no such scale (a non-finite value, or a spread
+// too small).
 __device__ __forceinline__ bool band_scale(unsigned max_o, unsigned min_o, float s, int* k) {
   const float top = unordered(max_o), bot = unordered(~min_o);
   *k = 0;
@@ -114,11 +122,21 @@ __device__ __forceinline__ bool band_scale(unsigned max_o, unsigned min_o, float
     return false;
   const double d = fmax((double)top - (double)s, (double)s - (double)bot);
   const double a = fmax(fabs((double)top), fabs((double)bot));
-  if (d == 0.0) return true;                     // every digit is zero whatever the scale (see q0)
+  if (d == 0.0) return true;                     // every digit is zero
   const int e = min(53 - ilogb(d), 60 - ilogb(a));
   if (e > 120) return false;
   *k = e;
   return true;
+}
+
+// y 2^k towards zero, |y| 2^k < 2^61: the significand from the word's top, shifted down.
+// (cvt.s64.f32 runs on the FP64 pipe and held it for a third of the kernel's time.)
+__device__ __forceinline__ long long to_fixed(float y, int k) {
+  const unsigned u = __float_as_uint(y);
+  const int down = min(189 - k - (int)((u >> 23) & 255u), 63);
+  const unsigned top = ((u << 7) & 0x3fffffffu) | 0x40000000u;
+  const long long q = (long long)(((unsigned long long)top << 32) >> down);
+  return (int)u < 0 ? -q : q;
 }
 
 __device__ __forceinline__ void ldsm4t(uint32_t (&r)[4], uint32_t addr) {
@@ -127,14 +145,14 @@ __device__ __forceinline__ void ldsm4t(uint32_t (&r)[4], uint32_t addr) {
 }
 __device__ __forceinline__ void mma16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0,
                                          uint32_t b1) {
-  asm volatile(
+  asm(
       "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
       "{%0,%1,%2,%3};"
       : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-// Two biased fixed-point values -> their seven digits as FP16 pairs, plane by plane.
+// Two biased fixed-point values -> their digits as FP16 pairs, plane by plane.
 // A byte u under the exponent byte 0x64 is the FP16 number 1024 + u.
 __device__ __forceinline__ void store_digits(__half* dst, unsigned long long ua,
                                              unsigned long long ub) {
@@ -153,9 +171,11 @@ __device__ __forceinline__ void store_digits(__half* dst, unsigned long long ua,
 }
 
 // Grid: x = partial slot (pixels N x / parts ..), y = tile of the upper block-triangle.
-// Bound: the tensor cores and the ldmatrix reads that feed them (a warp's 32 x 32
-// outputs: four reads of 512 bytes for eight MMAs).  Two CTAs share an SM, one's conversion
-// beside the other's products.
+// Bound: issue (half of the slots) and the latency of the shared-memory reads; the tensor
+// pipe is active 29% of the time, the ALU (digits, flushes) 46%.  A chunk's rows come by
+// asynchronous copies during the products of the one before, and 8 warps of 32 x 16 outputs
+// (128 registers) hide more latency than 4 of 32 x 32 (237): 350 x 350 x 188, with loads
+// into registers and 4 warps 1.02 ms, so 0.61.
 template <typename In>
 __global__ void __launch_bounds__(kThr, 2)
 k_syrk_digits(const In* __restrict__ cube, int64_t N, int B, int parts,
@@ -163,8 +183,9 @@ k_syrk_digits(const In* __restrict__ cube, int64_t N, int B, int parts,
               double* __restrict__ s1_part, double* __restrict__ s2_part,
               DevHeader* __restrict__ hdr) {
   extern __shared__ __align__(128) unsigned char smem[];
-  __half* blk[2] = {reinterpret_cast<__half*>(smem), reinterpret_cast<__half*>(smem + kBlockBytes)};
-  FxSync* sy = reinterpret_cast<FxSync*>(smem + 2 * kBlockBytes);
+  __half* blk = reinterpret_cast<__half*>(smem);                     // [2][kDigits][kPx][kRow]
+  unsigned char* raw = smem + 2 * kBlockBytes;                  // [2][kPx][raw_row]
+  FxSync* sy = reinterpret_cast<FxSync*>(raw + 2 * kPx * raw_row<In>());
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int g = blockIdx.x;
   int ti = 0, tj = blockIdx.y;                    // tile row by row
@@ -182,21 +203,18 @@ k_syrk_digits(const In* __restrict__ cube, int64_t N, int B, int parts,
     if (!band_scale(ext[b], ext[B + b], s, &k)) bad = 1;
     if (g == 0 && blockIdx.y == 0) shift_out[b] = s;
   }
-  {
+  if (tid < 2 * kTile) {
     const int h = tid >> 6, p = tid & 63;         // block, position in it
     const int b = (h ? tj : ti) * kTile + (p >> 1) + 32 * (p & 1);
-    int k = b == B ? 54 : 0;                      // the constant band: 64 * 2^48
-    float sc = 0.f;
+    int k = b == B ? 54 : 0;               // the constant band: D_0 = 64
     long long q0 = 0;
     if (b < B) {
       const float s = to_f32<In>(cube[b]);
       band_scale(ext[b], ext[B + b], s, &k);
-      sc = ext[b] == ~ext[B + b] ? 0.f : scalbnf(1.f, k);
-      q0 = __float2ll_rn(s * sc);
+      q0 = to_fixed(s, k);
     } else if (b == B) {
       q0 = -(64ll << 48);                         // digits of 0 - q0
     }
-    sy->scale[h][p] = sc;
     sy->q0[h][p] = q0;
     sy->k[h][p] = k;
     if (tid < 4) (&sy->used[0][0])[tid] = (&sy->used_b[0][0])[tid] = 0u;
@@ -207,49 +225,67 @@ k_syrk_digits(const In* __restrict__ cube, int64_t N, int B, int parts,
   }
 
   const int64_t n0 = N * g / parts, n1 = N * (g + 1) / parts;
-  const int m0 = (warp & 1) * 32, c0 = (warp >> 1) * 32;   // this warp's outputs
-  long long hi[2][4][4], lo[2][4][4];
+  const int m0 = (warp & 1) * 32, c0 = (warp >> 1) * 16;   // this warp's outputs
+  unsigned long long hi[2][2][4], lo[2][2][4];    // signed sums, modulo 2^64
+  unsigned long long hi_off = 0, lo_off = 0;         // what the magic numbers added
 #pragma unroll
   for (int i = 0; i < 2; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j)
+    for (int j = 0; j < 2; ++j)
 #pragma unroll
       for (int r = 0; r < 4; ++r) hi[i][j][r] = lo[i][j][r] = 0;
 
   // ldmatrix (transposed) addresses: A from [pixel][band] as 16 x 16, B as 16 x 16
-  const uint32_t sA = (uint32_t)__cvta_generic_to_shared(blk[0]) +
+  const uint32_t sA = (uint32_t)__cvta_generic_to_shared(blk) +
                       2u * (((lane & 7) + ((lane >> 4) & 1) * 8) * kRow + m0 + ((lane >> 3) & 1) * 8);
-  const uint32_t sB = (uint32_t)__cvta_generic_to_shared(blk[diag ? 0 : 1]) +
+  const uint32_t sB = (uint32_t)__cvta_generic_to_shared(blk) + (diag ? 0u : (uint32_t)kBlockBytes) +
                       2u * (((lane & 7) + ((lane >> 3) & 1) * 8) * kRow + c0 + ((lane >> 4) & 1) * 8);
 
   const int nconv = diag ? 1 : 2;
+  // the rows of a chunk, as the whole 16-byte units that hold them (the cube starts on one;
+  // the last one may end beyond it)
+  const int64_t cube_bytes = N * B * (int64_t)sizeof(In);
+  auto fetch = [&](int64_t c) {
+    constexpr int kUnits = raw_row<In>() / 16;
+    for (int e = tid; e < nconv * kPx * kUnits; e += kThr) {
+      const int h = e / (kPx * kUnits), p = e / kUnits % kPx, u = e % kUnits;
+      const int b0 = (h ? tj : ti) * kTile, nbands = min(kTile, B - b0);
+      if (c + p >= n1) continue;
+      const int64_t at = ((c + p) * B + b0) * (int64_t)sizeof(In);
+      const int64_t src = (at & ~(int64_t)15) + 16 * u;
+      if (src >= at + nbands * (int)sizeof(In)) continue;
+      const int bytes = cube_bytes - src < 16 ? (int)(cube_bytes - src) : 16;
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(
+                       (uint32_t)__cvta_generic_to_shared(raw + (h * kPx + p) * raw_row<In>() + 16 * u)),
+                   "l"(reinterpret_cast<const char*>(cube) + src), "r"(bytes)
+                   : "memory");
+    }
+  };
+  fetch(n0);
   int par = 0, since = 0;
   for (int64_t c = n0; c < n1; c += kPx, par ^= 1) {
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();               // the chunk has landed; the digits of the last one are read
     // conversion: warp = pixel, lane = bands lane and lane + 32 of the block
     for (int h = 0; h < nconv; ++h) {
-      const int b = (h ? tj : ti) * kTile + lane;
-      const bool inA = b < B, inB = b + 32 < B;
-      const float scA = sy->scale[h][2 * lane], scB = sy->scale[h][2 * lane + 1];
+      const int b0 = (h ? tj : ti) * kTile;
+      const bool inA = b0 + lane < B, inB = b0 + lane + 32 < B;
+      const int kA = sy->k[h][2 * lane], kB = sy->k[h][2 * lane + 1];
       const long long qA = sy->q0[h][2 * lane], qB = sy->q0[h][2 * lane + 1];
-      float va[kPx / 4], vb[kPx / 4];
-#pragma unroll
-      for (int u = 0; u < kPx / 4; ++u) {
-        const int64_t n = c + warp + 4 * u;
-        const In* row = cube + (n < n1 ? n : n0) * B + b;
-        va[u] = inA ? to_f32<In>(row[0]) : 0.f;
-        vb[u] = inB ? to_f32<In>(row[32]) : 0.f;
-      }
       unsigned long long used = 0;
 #pragma unroll
-      for (int u = 0; u < kPx / 4; ++u) {
-        const int p = warp + 4 * u;
+      for (int u = 0; u < kPx / 8; ++u) {
+        const int p = warp + 8 * u;
         unsigned long long ua = kBias, ub = kBias;
         if (c + p < n1) {
-          ua += (unsigned long long)(__float2ll_rn(va[u] * scA) - qA);
-          ub += (unsigned long long)(__float2ll_rn(vb[u] * scB) - qB);
+          const int skip = (int)((((c + p) * B + b0) * (int64_t)sizeof(In)) & 15);
+          const In* row = reinterpret_cast<const In*>(raw + (h * kPx + p) * raw_row<In>() + skip) + lane;
+          const float va = inA ? to_f32<In>(row[0]) : 0.f, vb = inB ? to_f32<In>(row[32]) : 0.f;
+          ua += (unsigned long long)(to_fixed(va, kA) - qA);
+          ub += (unsigned long long)(to_fixed(vb, kB) - qB);
         }
         used |= (ua ^ kBias) | (ub ^ kBias);
-        store_digits(blk[h] + (size_t)p * kRow + 2 * lane, ua, ub);
+        store_digits(blk + h * kBlockHalves + p * kRow + 2 * lane, ua, ub);
       }
       const unsigned ul = __reduce_or_sync(kFull, (unsigned)used);
       const unsigned uh = __reduce_or_sync(kFull, (unsigned)(used >> 32));
@@ -260,6 +296,7 @@ k_syrk_digits(const In* __restrict__ cube, int64_t N, int B, int parts,
       }
     }
     __syncthreads();
+    if (c + kPx < n1) fetch(c + kPx);   // beside the products
     auto digits = [](unsigned l, unsigned h) {   // how many digits, from the top, are not all zero
       return l ? kDigits - ((__ffs((int)l) - 1) >> 3) : (h ? 3 - ((__ffs((int)h) - 1) >> 3) : 0);
     };
@@ -268,14 +305,14 @@ k_syrk_digits(const In* __restrict__ cube, int64_t N, int B, int parts,
     if (tid < 2) sy->used[par ^ 1][tid] = sy->used_b[par ^ 1][tid] = 0u;
 
     // one level: all pairs of digits, then the sums into the integers with weight w
-    auto level = [&](int l, int w, long long (&tot)[2][4][4]) {
+    auto level = [&](int l, int w, auto& tot, unsigned long long& off) {
       const int ia = l - nbd + 1 > 0 ? l - nbd + 1 : 0, ib = l < na - 1 ? l : na - 1;
       if (ia > ib) return;
-      float acc[2][4][4];
+      float acc[2][2][4];
 #pragma unroll
       for (int i = 0; i < 2; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
+        for (int j = 0; j < 2; ++j)
 #pragma unroll
           for (int r = 0; r < 4; ++r) acc[i][j][r] = 0.f;
 #pragma unroll 1
@@ -284,58 +321,55 @@ k_syrk_digits(const In* __restrict__ cube, int64_t N, int B, int parts,
         const uint32_t pb = sB + (uint32_t)((l - i) * kPx * kRow * 2);
 #pragma unroll
         for (int ks = 0; ks < kPx / 16; ++ks) {
-          uint32_t a0[4], a1[4], b0[4], b1[4];
+          uint32_t a0[4], a1[4], b0[4];
           const uint32_t o = (uint32_t)(ks * 16 * kRow * 2);
           ldsm4t(a0, pa + o);
           ldsm4t(a1, pa + o + 32);
           ldsm4t(b0, pb + o);
-          ldsm4t(b1, pb + o + 32);
           mma16816(acc[0][0], a0, b0[0], b0[1]);
           mma16816(acc[0][1], a0, b0[2], b0[3]);
-          mma16816(acc[0][2], a0, b1[0], b1[1]);
-          mma16816(acc[0][3], a0, b1[2], b1[3]);
           mma16816(acc[1][0], a1, b0[0], b0[1]);
           mma16816(acc[1][1], a1, b0[2], b0[3]);
-          mma16816(acc[1][2], a1, b1[0], b1[1]);
-          mma16816(acc[1][3], a1, b1[2], b1[3]);
         }
       }
-      // |sum| <= 2^22: the low bits of 1.5 * 2^23 + sum are the integer
+      // |sum| <= 2^22: as an integer, the bits of 1.5 * 2^23 + sum are a constant + sum
+      off += 0x4B400000ull * (unsigned)w;
 #pragma unroll
       for (int i = 0; i < 2; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
+        for (int j = 0; j < 2; ++j)
 #pragma unroll
           for (int r = 0; r < 4; ++r)
-            tot[i][j][r] +=
-                (long long)(__float_as_int(__fadd_rn(acc[i][j][r], 12582912.f)) - 0x4B400000) * w;
+            tot[i][j][r] += (unsigned long long)__float_as_uint(__fadd_rn(acc[i][j][r], 12582912.f)) *
+                            (unsigned)w;
     };
     // levels 0 .. 3 in units of 2^72, levels 4 .. 7 in units of 2^40
 #pragma unroll 1
-    for (int l = 0; l < 4; ++l) level(l, 1 << (8 * (3 - l)), hi);
+    for (int l = 0; l < 4; ++l) level(l, 1 << (8 * (3 - l)), hi, hi_off);
 #pragma unroll 1
-    for (int l = 4; l < 8; ++l) level(l, 1 << (8 * (7 - l)), lo);
+    for (int l = 4; l < 8; ++l) level(l, 1 << (8 * (7 - l)), lo, lo_off);
     if (++since == 1 << 16) {      // |lo| < 2^62: carried over into hi
       since = 0;
 #pragma unroll
       for (int i = 0; i < 2; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
+        for (int j = 0; j < 2; ++j)
 #pragma unroll
           for (int r = 0; r < 4; ++r) {
-            hi[i][j][r] += lo[i][j][r] >> 32;
-            lo[i][j][r] &= 0xffffffffll;
+            lo[i][j][r] -= lo_off;
+            hi[i][j][r] += (unsigned long long)((long long)lo[i][j][r] >> 32);
+            lo[i][j][r] &= 0xffffffffull;
           }
+      lo_off = 0;
     }
-    __syncthreads();               // the digits are read; the next chunk may be written
   }
 
-  // pair sums in units of 2^(40 - k_a - k_b); a sum with the constant band is S1
+  // pair sums, in units of 2^(40 - k_a - k_b); a sum with the constant band is S1
   const int s2_elems = B * (B + 1) / 2;
 #pragma unroll
   for (int i = 0; i < 2; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j)
+    for (int j = 0; j < 2; ++j)
 #pragma unroll
       for (int r = 0; r < 4; ++r) {
         const int pr = m0 + 16 * i + (lane >> 2) + 8 * (r >> 1);
@@ -343,8 +377,9 @@ k_syrk_digits(const In* __restrict__ cube, int64_t N, int B, int parts,
         const int br = ti * kTile + (pr >> 1) + 32 * (pr & 1);
         const int bc = tj * kTile + (pc >> 1) + 32 * (pc & 1);
         if (br > bc || bc > B || br >= B) continue;   // below the diagonal, padding, (B, B)
-        const long long top = hi[i][j][r] + (lo[i][j][r] >> 32);
-        const double v = fma((double)top, 4294967296.0, (double)(lo[i][j][r] & 0xffffffffll));
+        const long long low = (long long)(lo[i][j][r] - lo_off);
+        const long long top = (long long)(hi[i][j][r] - hi_off) + (low >> 32);
+        const double v = fma((double)top, 4294967296.0, (double)(low & 0xffffffffll));
         const double x = ldexp(v, 40 - sy->k[0][pr] - sy->k[1][pc]);
         if (bc == B) s1_part[(size_t)g * B + br] = x;
         else s2_part[(size_t)g * s2_elems + packed_index(br, bc, B)] = x;
@@ -360,7 +395,7 @@ cudaError_t digits_typed(const In* cube, int64_t N, int B, float* shift, double*
   const int grid = (int)std::min<int64_t>(4 * device_sms(), (N + 31) / 32);
   k_band_range<In><<<grid, 256, 0, st>>>(cube, N, B, ext);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  const size_t smem = 2 * kBlockBytes + sizeof(FxSync);
+  const size_t smem = 2 * kBlockBytes + 2 * kPx * raw_row<In>() + sizeof(FxSync);
   auto kern = k_syrk_digits<In>;
   e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -385,8 +420,8 @@ cudaError_t launch_syrk_digits(const void* cube, pca_dtype dt, int64_t N, int B,
     case PCA_F32:
       return digits_typed((const float*)cube, N, B, shift, s1_part, s2_part, parts, ext, hdr, st);
     case PCA_BF16:
-      return digits_typed((const __nv_bfloat16*)cube, N, B, shift, s1_part, s2_part, parts, ext, hdr,
-                          st);
+      return digits_typed((const __nv_bfloat16*)cube, N, B, shift, s1_part, s2_part, parts, ext,
+                          hdr, st);
     case PCA_F16:
       return digits_typed((const __half*)cube, N, B, shift, s1_part, s2_part, parts, ext, hdr, st);
   }
