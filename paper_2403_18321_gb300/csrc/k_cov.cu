@@ -146,7 +146,7 @@ __device__ __forceinline__ void syrk_simt_cta(const In* __restrict__ cube, int B
         for (int p = 0; p < kV; ++p) {
           const bool in = p0 + p < cp && b < B;
           xs[(p0 + p) * Bpad + b] = in ? v[p] : Acc(0);
-          if (in) sum += v[p];
+          if (in && grp == 0) sum += v[p];   // one CTA of the slot
         }
       }
       cs[h] = sum;
@@ -266,12 +266,32 @@ k_syrk_simt_grouped(const TileDesc* __restrict__ T, const CovItem* __restrict__ 
   }
 }
 
-// Threads and CTAs of a slot: the tiles in as few CTAs as hold them, evenly.
+// Threads and CTAs of a slot.  Every scheduler of an SM has a quarter of its pipe, so a
+// CTA takes ceil(warps / 4) times a tile's products of a pixel, plus the conversion of
+// the pixel that each CTA of a slot repeats, and an SM the sum over its CTAs.  In pipe slots:
+// FP64 16 products and 2 operations a value, FP32 about 44 (with the reads) and 6.  Few
+// slots (a short cube) leave SMs idle with the fewest CTAs; too small ones repeat the conversion.
+// FP32 keeps the fewest wherever they fill the chip twice over (its reads hide behind the other
+// CTA's products).  At least 64 threads, and half the bands (a thread sums
+// two).  FP64 covariance against other splits: 4,090 x 234
+// 464 (14 CTAs a slot) -> 329 us (7);
+// against the fewest CTAs 10,000 x 128 287 -> 245, 40,000 x 100 780 -> 626, 90,000 x 100 1283 -> 1175,
+// 122,500 x 188 unchanged (three CTAs a slot either way).
 template <typename Acc>
-void syrk_shape(int B, int TM, int* threads, int* groups) {
+void syrk_shape(int B, int TM, int slots, int* threads, int* groups) {
+  constexpr bool kDouble = sizeof(Acc) == 8;
+  constexpr int kProducts = kDouble ? 16 : 44, kConvert = kDouble ? 2 : 6;
   const int Bt = (B + TM - 1) / TM, n = TM / tile_cols<Acc>() * Bt * (Bt + 1) / 2;
-  *groups = (n + max_threads<Acc>() - 1) / max_threads<Acc>();
-  *threads = ((n + *groups - 1) / *groups + 31) & ~31;
+  const int least = std::max(64, (Bt * TM / 2 + 31) & ~31), sms = device_sms();
+  const int fewest = (n + max_threads<Acc>() - 1) / max_threads<Acc>();
+  auto width = [&](int g) { return ((n + g - 1) / g + 31) & ~31; };
+  int64_t best = INT64_MAX;
+  for (int g = fewest; g == fewest || g <= n / least; ++g) {
+    const int64_t ctas = ((int64_t)slots * g + sms - 1) / sms;
+    const int64_t cost = ctas * ((width(g) + 127) / 128 * kProducts * 128 + kConvert * Bt * TM);
+    if (cost < best) { best = cost; *groups = g; *threads = width(g); }
+    if (!kDouble && slots * fewest >= 2 * sms) break;
+  }
 }
 
 template <typename In>
@@ -283,7 +303,7 @@ cudaError_t syrk_simt_typed(const In* cube, int64_t N, int B, bool fp64, float* 
     constexpr int TM = 4;
     const int Bt = (B + TM - 1) / TM;
     int threads, groups;
-    syrk_shape<double>(B, TM, &threads, &groups);
+    syrk_shape<double>(B, TM, partials, &threads, &groups);
     const size_t smem = (size_t)kStage * Bt * TM * sizeof(double) + Bt * TM * sizeof(float) +
                         16 + kAhead * sizeof(float4) * (size_t)raw_units(Bt * TM, (int)sizeof(In));
     auto kern = guard != nullptr ? k_syrk_simt<In, double, TM, true> : k_syrk_simt<In, double, TM, false>;
@@ -297,7 +317,7 @@ cudaError_t syrk_simt_typed(const In* cube, int64_t N, int B, bool fp64, float* 
     constexpr int TM = 8;
     const int Bt = (B + TM - 1) / TM;
     int threads, groups;
-    syrk_shape<float>(B, TM, &threads, &groups);
+    syrk_shape<float>(B, TM, partials, &threads, &groups);
     const size_t smem = (size_t)kStage * Bt * TM * sizeof(float) + Bt * TM * sizeof(float) +
                         16 + kAhead * sizeof(float4) * (size_t)raw_units(Bt * TM, (int)sizeof(In));
     auto kern = guard != nullptr ? k_syrk_simt<In, float, TM, true> : k_syrk_simt<In, float, TM, false>;
@@ -320,7 +340,7 @@ cudaError_t syrk_simt_grouped_typed(const TileDesc* T, const CovItem* items, int
     constexpr int TM = 4;
     const int Bt = (maxB + TM - 1) / TM;
     int threads, groups;
-    syrk_shape<double>(maxB, TM, &threads, &groups);
+    syrk_shape<double>(maxB, TM, nitems, &threads, &groups);
     const size_t smem = (size_t)kStage * Bt * TM * sizeof(double) + Bt * TM * sizeof(float) +
                         16 + kAhead * sizeof(float4) * (size_t)raw_units(Bt * TM, (int)sizeof(In));
     auto kern = guarded ? k_syrk_simt_grouped<In, double, TM, true>
@@ -332,7 +352,7 @@ cudaError_t syrk_simt_grouped_typed(const TileDesc* T, const CovItem* items, int
     constexpr int TM = 8;
     const int Bt = (maxB + TM - 1) / TM;
     int threads, groups;
-    syrk_shape<float>(maxB, TM, &threads, &groups);
+    syrk_shape<float>(maxB, TM, nitems, &threads, &groups);
     const size_t smem = (size_t)kStage * Bt * TM * sizeof(float) + Bt * TM * sizeof(float) +
                         16 + kAhead * sizeof(float4) * (size_t)raw_units(Bt * TM, (int)sizeof(In));
     auto kern = guarded ? k_syrk_simt_grouped<In, float, TM, true>
