@@ -146,7 +146,9 @@ __device__ __forceinline__ void syrk_simt_cta(const In* __restrict__ cube, int B
         for (int p = 0; p < kV; ++p) {
           const bool in = p0 + p < cp && b < B;
           xs[(p0 + p) * Bpad + b] = in ? v[p] : Acc(0);
-          if (in && grp == 0) sum += v[p];   // one CTA of the slot
+          // S1 is one CTA's of the slot; in FP32, where the addition is cheap, the test
+          // itself cost more (610 x 340 x 103: 236 us with it, 205 without)
+          if (in && (sizeof(Acc) == 4 || grp == 0)) sum += v[p];
         }
       }
       cs[h] = sum;
@@ -271,12 +273,11 @@ k_syrk_simt_grouped(const TileDesc* __restrict__ T, const CovItem* __restrict__ 
 // the pixel that each CTA of a slot repeats, and an SM the sum over its CTAs.  In pipe slots:
 // FP64 16 products and 2 operations a value, FP32 about 44 (with the reads) and 6.  Few
 // slots (a short cube) leave SMs idle with the fewest CTAs; too small ones repeat the conversion.
-// FP32 keeps the fewest wherever they fill the chip twice over (its reads hide behind the other
-// CTA's products).  At least 64 threads, and half the bands (a thread sums
-// two).  FP64 covariance against other splits: 4,090 x 234
-// 464 (14 CTAs a slot) -> 329 us (7);
-// against the fewest CTAs 10,000 x 128 287 -> 245, 40,000 x 100 780 -> 626, 90,000 x 100 1283 -> 1175,
-// 122,500 x 188 unchanged (three CTAs a slot either way).
+// FP32 keeps the fewest wherever they fill the chip twice over (its reads hide behind the
+// other CTA's products).  At least 64 threads, and half the bands (a thread sums two).
+// FP64 covariance of 4,090 x 234: 14 CTAs a slot 464 us, 7 (chosen) 329; against the
+// fewest CTAs 10,000 x 128 287 -> 245 us, 40,000 x 100 780 -> 626, 90,000 x 100 1283 ->
+// 1175, 122,500 x 188 unchanged (three CTAs a slot either way).
 template <typename Acc>
 void syrk_shape(int B, int TM, int slots, int* threads, int* groups) {
   constexpr bool kDouble = sizeof(Acc) == 8;
