@@ -172,7 +172,7 @@ __device__ __forceinline__ void store_digits(__half* dst, unsigned long long ua,
 
 // Grid: x = partial slot (pixels N x / parts ..), y = tile of the upper block-triangle.
 // Bound: issue (half of the slots) and the latency of the shared-memory reads; the tensor
-// pipe is active 29% of the time, the ALU (digits, flushes) 46%.  A chunk's rows come by
+// pipe is active 29% of the time, the ALU (conversion, digits) 55%.  A chunk's rows come by
 // asynchronous copies during the products of the one before, and 8 warps of 32 x 16 outputs
 // (128 registers) hide more latency than 4 of 32 x 32 (237): 350 x 350 x 188, with loads
 // into registers and 4 warps 1.02 ms, so 0.61.
