@@ -8,11 +8,12 @@
 // products are exact: Ozaki, Ogita, Oishi and Rump, Numer. Algorithms 59, 2012).
 // Digits are exact in FP16, a product of two is at most 2^14, and the sums over a chunk of
 // 32 pixels of all pairs (i, j) of one level i + j stay below 2^22: exact in the FP32
-// accumulators.  They are then added as 64-bit integers, and a partial is rounded once.
-// Levels 0 .. 7 are formed; what is left out of a product is below 2^-57 of the largest
-// |x_a| |x_b| (an FP64 sum rounds to 2^-53 of itself at every pixel).  Digits that
-// are zero throughout a chunk are skipped: FP32 cubes have four to six that are not, 16-bit
-// ones two to four.
+// accumulators.  They are then added as integers of 64 bits in three units, and a
+// partial is rounded at its end.  All levels, 0 .. 12, are formed: the scale follows the
+// band's farthest value, so that beside a hot or no-data pixel the products of all others
+// lie in the low levels (without levels 8 .. 12 one pixel of 9999 among 10^6 in [0, 1)
+// cost the variance 2e-13 of itself).  Digits that are zero throughout a chunk are skipped:
+// FP32 cubes have four to six that are not, 16-bit ones two to four.
 //
 //   k_band_range     largest and smallest value of every band (one pass)
 //   k_syrk_digits    one CTA = one 64 x 64 band tile of one pixel range
@@ -227,13 +228,17 @@ k_syrk_digits(const In* __restrict__ cube, int64_t N, int B, int parts,
   const int64_t n0 = N * g / parts, n1 = N * (g + 1) / parts;
   const int m0 = (warp & 1) * 32, c0 = (warp >> 1) * 16;   // this warp's outputs
   unsigned long long hi[2][2][4], lo[2][2][4];    // signed sums, modulo 2^64
-  unsigned long long hi_off = 0, lo_off = 0;         // what the magic numbers added
+  unsigned long long hi_off = 0, lo_off = 0, ex_off = 0;   // what the magic numbers added
+  // levels 8 .. 12, in units of 1: few chunks have them, so they stay in local memory
+  // (volatile: the registers hold hi and lo)
+  volatile unsigned long long ex[16];
+  bool ex_used = false;
 #pragma unroll
   for (int i = 0; i < 2; ++i)
 #pragma unroll
     for (int j = 0; j < 2; ++j)
 #pragma unroll
-      for (int r = 0; r < 4; ++r) hi[i][j][r] = lo[i][j][r] = 0;
+      for (int r = 0; r < 4; ++r) hi[i][j][r] = lo[i][j][r] = ex[8 * i + 4 * j + r] = 0;
 
   // ldmatrix (transposed) addresses: A from [pixel][band] as 16 x 16, B as 16 x 16
   const uint32_t sA = (uint32_t)__cvta_generic_to_shared(blk) +
@@ -262,6 +267,20 @@ k_syrk_digits(const In* __restrict__ cube, int64_t N, int B, int parts,
     }
   };
   fetch(n0);
+  // |ex| < 2^63: what is above its 40 low bits goes over to lo
+  auto carry_ex = [&]() {
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int j = 0; j < 2; ++j)
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          const unsigned long long e = ex[8 * i + 4 * j + r] - ex_off;
+          lo[i][j][r] += (unsigned long long)((long long)e >> 40);
+          ex[8 * i + 4 * j + r] = e & 0xffffffffffull;
+        }
+    ex_off = 0;
+  };
   int par = 0, since = 0;
   for (int64_t c = n0; c < n1; c += kPx, par ^= 1) {
     asm volatile("cp.async.wait_all;" ::: "memory");
@@ -304,10 +323,10 @@ k_syrk_digits(const In* __restrict__ cube, int64_t N, int B, int parts,
     const int nbd = diag ? na : digits(sy->used_b[par][0], sy->used_b[par][1]);
     if (tid < 2) sy->used[par ^ 1][tid] = sy->used_b[par ^ 1][tid] = 0u;
 
-    // one level: all pairs of digits, then the sums into the integers with weight w
-    auto level = [&](int l, int w, auto& tot, unsigned long long& off) {
+    // one level: all pairs of digits, then the sums into the integers by add(i, j, r, bits)
+    auto level = [&](int l, auto add) {
       const int ia = l - nbd + 1 > 0 ? l - nbd + 1 : 0, ib = l < na - 1 ? l : na - 1;
-      if (ia > ib) return;
+      if (ia > ib) return false;
       float acc[2][2][4];
 #pragma unroll
       for (int i = 0; i < 2; ++i)
@@ -333,22 +352,40 @@ k_syrk_digits(const In* __restrict__ cube, int64_t N, int B, int parts,
         }
       }
       // |sum| <= 2^22: as an integer, the bits of 1.5 * 2^23 + sum are a constant + sum
-      off += 0x4B400000ull * (unsigned)w;
 #pragma unroll
       for (int i = 0; i < 2; ++i)
 #pragma unroll
         for (int j = 0; j < 2; ++j)
 #pragma unroll
           for (int r = 0; r < 4; ++r)
-            tot[i][j][r] += (unsigned long long)__float_as_uint(__fadd_rn(acc[i][j][r], 12582912.f)) *
-                            (unsigned)w;
+            add(i, j, r, (unsigned long long)__float_as_uint(__fadd_rn(acc[i][j][r], 12582912.f)));
+      return true;
     };
-    // levels 0 .. 3 in units of 2^72, levels 4 .. 7 in units of 2^40
+    // levels 0 .. 3 in units of 2^72, 4 .. 7 in units of 2^40, 8 .. 12 in units of 1
 #pragma unroll 1
-    for (int l = 0; l < 4; ++l) level(l, 1 << (8 * (3 - l)), hi, hi_off);
+    for (int l = 0; l < 4; ++l) {
+      const unsigned w = 1u << (8 * (3 - l));
+      if (level(l, [&](int i, int j, int r, unsigned long long b) { hi[i][j][r] += b * w; }))
+        hi_off += 0x4B400000ull * w;
+    }
 #pragma unroll 1
-    for (int l = 4; l < 8; ++l) level(l, 1 << (8 * (7 - l)), lo, lo_off);
-    if (++since == 1 << 16) {      // |lo| < 2^62: carried over into hi
+    for (int l = 4; l < 8; ++l) {
+      const unsigned w = 1u << (8 * (7 - l));
+      if (level(l, [&](int i, int j, int r, unsigned long long b) { lo[i][j][r] += b * w; }))
+        lo_off += 0x4B400000ull * w;
+    }
+#pragma unroll 1
+    for (int l = 8; l < na + nbd - 1; ++l) {
+      const int sh = 8 * (12 - l);
+      level(l, [&](int i, int j, int r, unsigned long long b) {
+        ex[8 * i + 4 * j + r] = ex[8 * i + 4 * j + r] + (b << sh);
+      });
+      ex_off += 0x4B400000ull << sh;
+      ex_used = true;
+    }
+    ++since;
+    if (ex_used && (since & 255) == 0) carry_ex();
+    if (since == 1 << 16) {        // |lo| < 2^63: carried over into hi
       since = 0;
 #pragma unroll
       for (int i = 0; i < 2; ++i)
@@ -364,7 +401,8 @@ k_syrk_digits(const In* __restrict__ cube, int64_t N, int B, int parts,
     }
   }
 
-  // pair sums, in units of 2^(40 - k_a - k_b); a sum with the constant band is S1
+  if (ex_used) carry_ex();
+  // pair sums, in units of 2^(-k_a - k_b); a sum with the constant band is S1
   const int s2_elems = B * (B + 1) / 2;
 #pragma unroll
   for (int i = 0; i < 2; ++i)
@@ -379,8 +417,16 @@ k_syrk_digits(const In* __restrict__ cube, int64_t N, int B, int parts,
         if (br > bc || bc > B || br >= B) continue;   // below the diagonal, padding, (B, B)
         const long long low = (long long)(lo[i][j][r] - lo_off);
         const long long top = (long long)(hi[i][j][r] - hi_off) + (low >> 32);
-        const double v = fma((double)top, 4294967296.0, (double)(low & 0xffffffffll));
-        const double x = ldexp(v, 40 - sy->k[0][pr] - sy->k[1][pc]);
+        // the magnitude of top 2^72 + low 2^40 + ex, rounded to FP64 twice at most
+        unsigned long long t = (unsigned long long)top, m = (unsigned long long)low & 0xffffffffull;
+        unsigned long long f = ex_used ? ex[8 * i + 4 * j + r] : 0ull;
+        if (top < 0) {
+          f = (0ull - f) & 0xffffffffffull;
+          m = ((f != 0 ? ~m : 0ull - m)) & 0xffffffffull;
+          t = (f | m) != 0 ? ~t : 0ull - t;
+        }
+        const double v = fma((double)t, 4294967296.0, fma((double)f, 0x1p-40, (double)m));
+        const double x = ldexp(top < 0 ? -v : v, 40 - sy->k[0][pr] - sy->k[1][pc]);
         if (bc == B) s1_part[(size_t)g * B + br] = x;
         else s2_part[(size_t)g * s2_elems + packed_index(br, bc, B)] = x;
       }
