@@ -104,10 +104,8 @@ Layout make_layout(int64_t N, int B, int k, pca_dtype dt, pca_precision prec, in
     L.s2_bytes_el = 4;
   } else {
     L.partials = (int)std::min<int64_t>(kMaxPartials, std::max<int64_t>(1, (N + 255) / 256));
-    if (prec == PCA_PREC_P64) L.dig_parts = syrk_digits_parts(N, B, num_sms);
     L.s2_bytes_el = prec == PCA_PREC_P64 ? 8 : 4;
   }
-  const size_t slots = (size_t)std::max(L.partials, L.dig_parts);
   L.s2_elems = B * (B + 1) / 2;
   const size_t BB8 = sizeof(double) * (size_t)B * B;
   size_t o = 0;
@@ -115,9 +113,8 @@ Layout make_layout(int64_t N, int B, int k, pca_dtype dt, pca_precision prec, in
   L.hdr = take(sizeof(DevHeader));
   L.shift = take(sizeof(float) * B);
   L.escale = take(sizeof(int) * B);
-  L.ext = take(sizeof(unsigned) * 2 * B);
-  L.s1_part = take(sizeof(double) * slots * B);
-  L.s2_part = take((size_t)L.s2_bytes_el * slots * L.s2_elems);
+  L.s1_part = take(sizeof(double) * (size_t)L.partials * B);
+  L.s2_part = take((size_t)L.s2_bytes_el * L.partials * L.s2_elems);
   L.dvec = take(sizeof(double) * B);
   L.cov = take(BB8);
   L.cdf = take(BB8);
@@ -228,7 +225,6 @@ struct Ptrs {
   DevHeader* hdr;
   float* shift;
   int* escale;
-  unsigned* ext;
   double* s1p;
   void* s2p;
   double* dvec;
@@ -259,7 +255,6 @@ Ptrs carve(void* workspace, const Layout& L) {
   p.hdr = reinterpret_cast<DevHeader*>(ws + L.hdr);
   p.shift = reinterpret_cast<float*>(ws + L.shift);
   p.escale = reinterpret_cast<int*>(ws + L.escale);
-  p.ext = reinterpret_cast<unsigned*>(ws + L.ext);
   p.s1p = reinterpret_cast<double*>(ws + L.s1_part);
   p.s2p = ws + L.s2_part;
   p.dvec = reinterpret_cast<double*>(ws + L.dvec);
@@ -294,7 +289,8 @@ cudaError_t run_cov(const void* cube, pca_dtype dt, int64_t N, int B, pca_precis
                     const Layout& L, const Ptrs& P, double* mu, cudaStream_t st, StageMark& pm,
                     bool digits = false) {
   cudaError_t e;
-  const int parts = digits ? L.dig_parts : L.partials;
+  int parts = L.partials;
+  const int* simt = nullptr;   // digits: set when the FP64 SIMT form has made the partials
   pm.mark(0);
   if (prec == PCA_PREC_MIX) {
     e = launch_syrk_tc(cube, dt, N, B, P.shift, P.escale, P.s1p, (float*)P.s2p, L.partials,
@@ -305,16 +301,21 @@ cudaError_t run_cov(const void* cube, pca_dtype dt, int64_t N, int B, pca_precis
     e = launch_syrk_simt(cube, dt, N, B, false, P.shift, P.s1p, P.s2p, L.partials, st,
                          &P.hdr->cov_range, P.escale);
   } else if (digits) {
-    e = launch_syrk_digits(cube, dt, N, B, P.shift, P.s1p, (double*)P.s2p, parts, P.ext, P.hdr, st);
+    // the band ranges lie where an eigen-solve would have its vectors
+    parts = syrk_digits_parts(B, device_sms(), L.partials);
+    e = launch_syrk_digits(cube, dt, N, B, P.shift, P.s1p, (double*)P.s2p, parts,
+                           reinterpret_cast<unsigned*>(P.vc), P.hdr, st);
     if (e != cudaSuccess) return e;
-    e = launch_syrk_simt(cube, dt, N, B, true, P.shift, P.s1p, P.s2p, parts, st, &P.hdr->fx_range);
+    simt = &P.hdr->fx_range;
+    e = launch_syrk_simt(cube, dt, N, B, true, P.shift, P.s1p, P.s2p, L.partials, st, simt);
   } else {
-    e = launch_syrk_simt(cube, dt, N, B, prec == PCA_PREC_P64, P.shift, P.s1p, P.s2p, parts, st);
+    e = launch_syrk_simt(cube, dt, N, B, prec == PCA_PREC_P64, P.shift, P.s1p, P.s2p, L.partials, st);
   }
   if (e != cudaSuccess) return e;
   pm.mark(1);
   return launch_cov_finalize(P.shift, P.s1p, P.s2p, L.s2_bytes_el == 8, parts, N, B, mu, P.C,
-                             P.muf, P.dvec, P.hdr, st, prec == PCA_PREC_MIX ? P.escale : nullptr);
+                             P.muf, P.dvec, P.hdr, st, prec == PCA_PREC_MIX ? P.escale : nullptr,
+                             simt, L.partials);
 }
 
 // stage 4: Jacobi (rotating V), FP64 refinement, sort and sign rule

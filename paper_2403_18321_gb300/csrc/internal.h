@@ -36,11 +36,10 @@ struct DevHeader {
 
 // Offsets (bytes) of every workspace region; all 256-byte aligned.
 struct Layout {
-  size_t hdr, shift, escale, ext, s1_part, s2_part, dvec, cov, cdf, rank, sgn, diag32, v32, lam, vc, w, s, r, e, vk, muf;
+  size_t hdr, shift, escale, s1_part, s2_part, dvec, cov, cdf, rank, sgn, diag32, v32, lam, vc, w, s, r, e, vk, muf;
   size_t ptc_shift, ptc_escale, ptc_planes, ptc_colscale, ptc_corr;   // tensor-core projection
   size_t total;
   int partials;      // number of covariance partial slots the SYRK uses
-  int dig_parts;     // P64: partial slots of the covariance call's digit products
   int tc_ctas;       // MIX: CTAs of the tensor-core pass (partials spread over them)
   int s2_elems;      // packed upper-triangle entries per partial: B(B+1)/2
   int s2_bytes_el;   // 4 (FP32 partials) or 8 (FP64 partials)
@@ -160,10 +159,10 @@ cudaError_t launch_syrk_simt(const void* cube, pca_dtype dt, int64_t N, int B, b
                              float* shift, double* s1_part, void* s2_part, int partials,
                              cudaStream_t st, const int* guard = nullptr, int* escale = nullptr);
 
-// FP64 covariance partials from exact products of 8-bit digits on the tensor cores;
-// ext: 2 B words of scratch.  A band without a fixed-point form sets hdr->fx_range, and
+// FP64 covariance partials from exact products of 8-bit digits on the tensor cores, in at
+// most max_parts slots; ext: 2 B words of scratch.  A band without a fixed-point form sets hdr->fx_range, and
 // the caller's guarded SIMT launch forms the partials.
-int syrk_digits_parts(int64_t N, int B, int num_sms);   // partial slots
+int syrk_digits_parts(int B, int num_sms, int max_parts);   // partial slots
 cudaError_t launch_syrk_digits(const void* cube, pca_dtype dt, int64_t N, int B, float* shift,
                                double* s1_part, double* s2_part, int parts, unsigned* ext,
                                DevHeader* hdr, cudaStream_t st);
@@ -186,10 +185,12 @@ bool syrk_tc_supported(int B);
 // Sums the partials, applies the shift correction, writes mu (FP64), C (FP64, full
 // symmetric) and mu_f (FP32), flags non-finite sums in the header.
 // escale (nullable): S2 partials are scaled by 2^(escale[i] + escale[j]).
+// alt (nullable): a device word; where it is not zero there are alt_partials partials.
 cudaError_t launch_cov_finalize(const float* shift, const double* s1_part, const void* s2_part,
                                 bool fp64_partials, int partials, int64_t N, int B, double* mu,
                                 double* C, float* mu_f, double* dvec, DevHeader* hdr,
-                                cudaStream_t st, const int* escale = nullptr);
+                                cudaStream_t st, const int* escale = nullptr,
+                                const int* alt = nullptr, int alt_partials = 0);
 
 // FP32 odd-even Jacobi on one thread-block cluster: writes diag32 [B'] and V32
 // [B'][B'].  relative_stop selects the element-wise relative stop test (else

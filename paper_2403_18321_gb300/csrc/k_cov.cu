@@ -388,8 +388,10 @@ __device__ __forceinline__ void s1_reduce_band(int b, const double* __restrict__
 __global__ void k_s1_reduce(const double* __restrict__ s1_part, int partials, int B, int64_t N,
                             const float* __restrict__ shift, double* __restrict__ dvec,
                             double* __restrict__ mu, float* __restrict__ mu_f,
-                            DevHeader* __restrict__ hdr) {
+                            DevHeader* __restrict__ hdr, const int* __restrict__ alt,
+                            int alt_partials) {
   pdl_begin();
+  if (alt != nullptr && *alt != 0) partials = alt_partials;
   s1_reduce_band(blockIdx.x, s1_part, partials, B, N, shift, dvec, mu, mu_f, hdr);
 }
 __global__ void k_s1_reduce_batched(const TileDesc* __restrict__ T) {
@@ -467,8 +469,10 @@ template <typename Acc>
 __global__ void __launch_bounds__(kFinWarps * 32)
 k_cov_finalize(const Acc* __restrict__ s2_part, int partials, int s2_elems, int B, int64_t N,
                const double* __restrict__ dvec, double* __restrict__ C,
-               DevHeader* __restrict__ hdr, const int* __restrict__ escale) {
+               DevHeader* __restrict__ hdr, const int* __restrict__ escale,
+               const int* __restrict__ alt, int alt_partials) {
   pdl_begin();
+  if (alt != nullptr && *alt != 0) partials = alt_partials;
   cov_finalize_block<Acc>(blockIdx.x, s2_part, partials, s2_elems, B, N, dvec, C, hdr, escale);
 }
 template <typename Acc>
@@ -503,17 +507,18 @@ cudaError_t launch_syrk_simt(const void* cube, pca_dtype dt, int64_t N, int B, b
 cudaError_t launch_cov_finalize(const float* shift, const double* s1_part, const void* s2_part,
                                 bool fp64_partials, int partials, int64_t N, int B, double* mu,
                                 double* C, float* mu_f, double* dvec, DevHeader* hdr,
-                                cudaStream_t st, const int* escale) {
-  const cudaError_t e =
-      launch_after(k_s1_reduce, B, 32, 0, st, s1_part, partials, B, N, shift, dvec, mu, mu_f, hdr);
+                                cudaStream_t st, const int* escale, const int* alt,
+                                int alt_partials) {
+  const cudaError_t e = launch_after(k_s1_reduce, B, 32, 0, st, s1_part, partials, B, N, shift, dvec,
+                                     mu, mu_f, hdr, alt, alt_partials);
   if (e != cudaSuccess) return e;
   const int s2_elems = B * (B + 1) / 2;
   const int grid = (s2_elems + 31) / 32;
   if (fp64_partials)
     return launch_after(k_cov_finalize<double>, grid, kFinWarps * 32, 0, st, (const double*)s2_part,
-                        partials, s2_elems, B, N, dvec, C, hdr, escale);
+                        partials, s2_elems, B, N, dvec, C, hdr, escale, alt, alt_partials);
   return launch_after(k_cov_finalize<float>, grid, kFinWarps * 32, 0, st, (const float*)s2_part,
-                      partials, s2_elems, B, N, dvec, C, hdr, escale);
+                      partials, s2_elems, B, N, dvec, C, hdr, escale, alt, alt_partials);
 }
 
 cudaError_t launch_syrk_simt_grouped(const TileDesc* T, const CovItem* items, int nitems,

@@ -452,11 +452,14 @@ cudaError_t digits_typed(const In* cube, int64_t N, int B, float* shift, double*
 
 }  // namespace
 
-// Eight CTAs an SM (two at a time), a chunk of pixels at least.
-int syrk_digits_parts(int64_t N, int B, int num_sms) {
+// Eight CTAs an SM, two at a time.  Few bands or pixels: as many slots as the FP64 sums
+// have (one for 256 pixels, the workspace holds no more), less the start of a last round.
+int syrk_digits_parts(int B, int num_sms, int max_parts) {
   const int nb = (B + kTile) / kTile, tiles = nb * (nb + 1) / 2;
-  const int64_t cap = std::max(1, 8 * num_sms / tiles);
-  return (int)std::min<int64_t>(cap, std::max<int64_t>(1, (N + kPx - 1) / kPx));
+  const int parts = std::max(1, 8 * num_sms / tiles);
+  if (parts <= max_parts) return parts;
+  const int rounds = max_parts * tiles / (2 * num_sms);
+  return rounds > 0 ? std::max(1, rounds * 2 * num_sms / tiles) : max_parts;
 }
 
 cudaError_t launch_syrk_digits(const void* cube, pca_dtype dt, int64_t N, int B, float* shift,

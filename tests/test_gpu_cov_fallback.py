@@ -1,0 +1,34 @@
+"""The FP64 sums behind the digit products of a P64 covariance: a band without a
+fixed-point form gives the sums of a fit, slot by slot, and a workspace sized for more
+bands serves fewer."""
+import numpy as np
+import pytest
+import torch
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("N,B", [(3001, 17), (20_003, 60), (100_000, 256)])
+def test_fallback_sums_in_the_slots_of_a_fit(gbpca_lib, N, B):
+    Y = np.random.default_rng(B).uniform(0.0, 1.0, (N, B)).astype(np.float32)
+    Y[:, 3] *= np.float32(1e-37)       # no fixed-point scale: every band takes the FP64 sums
+    Yd = torch.from_numpy(Y).cuda()
+    mu, C, info = gbpca_lib.covariance(Yd, "p64")
+    fit = gbpca_lib.fit(Yd, 1, precision="p64", project=False)
+    assert info["status"] == 0
+    assert torch.equal(mu, fit[0])
+    lam = torch.linalg.eigvalsh(C).flip(0)
+    assert abs(lam[0].item() - fit[1][0].item()) <= 1e-12 * lam[0].item()
+
+
+@pytest.mark.gpu
+def test_workspace_of_more_bands_serves_fewer(gbpca_lib):
+    g = gbpca_lib
+    N = 20_000
+    ws = g.make_workspace(N, 128, 4, 0, "p64", torch.device("cuda"))
+    for B in (128, 63, 40):
+        Y = torch.rand(N, B, device="cuda")
+        _, C, info = g.covariance(Y, "p64", workspace=ws)
+        assert info["status"] == 0
+        ev = g.fit(Y, 4, precision="p64", workspace=ws)[1]
+        ref = torch.linalg.eigvalsh(C).flip(0)
+        assert (ev - ref).abs().max().item() <= 1e-10 * ref[0].item()
