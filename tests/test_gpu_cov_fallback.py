@@ -23,7 +23,7 @@ def test_fallback_sums_in_the_slots_of_a_fit(gbpca_lib, N, B):
 @pytest.mark.gpu
 def test_workspace_of_more_bands_serves_fewer(gbpca_lib):
     g = gbpca_lib
-    N = 20_000
+    N = 100_000
     ws = g.make_workspace(N, 128, 4, 0, "p64", torch.device("cuda"))
     for B in (128, 63, 40):
         Y = torch.rand(N, B, device="cuda")
