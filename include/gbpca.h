@@ -142,10 +142,14 @@ int pca_fit(const void *cube, pca_dtype dtype, int64_t N, int B, int k, double t
  *
  * pca_covariance -- Algorithm 1 stages 2-3: mu [B] and C = X^T X/(N-1),
  *   cov [B][B] FP64 row-major (full symmetric).  prec selects the
- *   covariance form (P64: exact products and sums of 56-bit fixed-point
- *   values, rounded to FP64 partials, where a fit adds in FP64; P32: FP32
- *   SIMT; MIX: split-FP16 tensor cores on per-band shifted and power-of-two
- *   scaled values).
+ *   covariance form (P64: exact products and sums of fixed-point values,
+ *   rounded to FP64 partials, where a fit adds in FP64.  The fixed point's
+ *   unit is at most 2^-53 of the largest distance of a value from the
+ *   first pixel's; where more than max(16, N / 4096) values of a band have
+ *   bits below it, or a band has no such form, all is added in FP64 as in a
+ *   fit; the bits cut off change C_ab by less than
+ *   2^-52 sqrt(2 max(16, N / 4096)) sqrt(C_aa C_bb).  P32: FP32 SIMT; MIX:
+ *   split-FP16 tensor cores on per-band shifted and power-of-two scaled values).
  * pca_eigh -- Algorithm 1 stage 4 on a given symmetric matrix A [B][B] FP64
  *   (device): cyclic Jacobi (Eqs. 2-10), FP64 refinement (P32: none; MIX: one
  *   iteration and two orthogonalisation steps; P64: five and three),

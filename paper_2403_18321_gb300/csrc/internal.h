@@ -160,8 +160,8 @@ cudaError_t launch_syrk_simt(const void* cube, pca_dtype dt, int64_t N, int B, b
                              cudaStream_t st, const int* guard = nullptr, int* escale = nullptr);
 
 // FP64 covariance partials from exact products of 8-bit digits on the tensor cores, in at
-// most max_parts slots; ext: 2 B words of scratch.  A band without a fixed-point form sets hdr->fx_range, and
-// the caller's guarded SIMT launch forms the partials.
+// most max_parts slots; ext: 3 B words of scratch.  A band without a fixed-point form that
+// holds its values sets hdr->fx_range, and the caller's guarded SIMT launch forms the partials.
 int syrk_digits_parts(int B, int num_sms, int max_parts);   // partial slots
 cudaError_t launch_syrk_digits(const void* cube, pca_dtype dt, int64_t N, int B, float* shift,
                                double* s1_part, double* s2_part, int parts, unsigned* ext,

@@ -19,7 +19,13 @@
 //   k_syrk_digits    one CTA = one 64 x 64 band tile of one pixel range
 // The fixed-point scale of a band comes from its range.  A band with a non-finite value
 // or a spread too small for an FP32 scale sets hdr->fx_range, and the FP64 SIMT
-// form (guarded by it) does the work.
+// form (guarded by it) does the work.  So does a band of which more than lost_max values have
+// bits below the scale's unit u, which is at most 2^-53 of the distance d of two of its
+// values (values below 2^-30 of the farthest one; their bits are cut off).  n such values
+// move a covariance by at most u sqrt(n) of sqrt(C_bb / (N - 1)), and C_aa (N - 1) >= d^2 / 2:
+// 2^-52 sqrt(2 n) of sqrt(C_aa C_bb) for both factors.  lost_max = N / 4096 (16 at least) makes
+// that sqrt(N / 2) 2^-57 at its worst (1.3e-15 at 16 values, 5e-15 at 10^6 pixels), and lets
+// the few values near zero of a cube with no-data pixels pass.
 //
 // The covariance call, FP64 products -> these: 350 x 350 x 188 FP32 4.74 -> 0.61 ms,
 // 610 x 340 x 103 2.88 -> 0.51, 512 x 512 x 224 BF16 13.7 -> 1.22, 10,000 x 50 0.189 -> 0.058.
@@ -70,7 +76,8 @@ __device__ __forceinline__ float unordered(unsigned o) {
   return __uint_as_float(o & 0x80000000u ? o ^ 0x80000000u : ~o);
 }
 
-// ext[b] = max of ordered(y_b), ext[B + b] = max of ~ordered(y_b); both start at 0.
+// ext[b] = max of ordered(y_b), ext[B + b] = max of ~ordered(y_b); ext[2 B + b], filled by
+// k_syrk_digits, counts the values with lost bits.  All start at 0.
 // Bound: the read of the cube.  Warp = pixel, lane = bands lane, lane + 32, ...
 template <typename In>
 __global__ void __launch_bounds__(256)
@@ -140,6 +147,13 @@ __device__ __forceinline__ long long to_fixed(float y, int k) {
   return (int)u < 0 ? -q : q;
 }
 
+// Whether y has bits that to_fixed cuts off: its lowest set bit against the shift.
+__device__ __forceinline__ bool loses_bits(float y, int k) {
+  const unsigned u = __float_as_uint(y);
+  const unsigned top = (u << 7) | 0x40000000u;
+  return y != 0.f && 189 - k - (int)((u >> 23) & 255u) > 31 + __ffs((int)top);
+}
+
 __device__ __forceinline__ void ldsm4t(uint32_t (&r)[4], uint32_t addr) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
@@ -180,7 +194,7 @@ __device__ __forceinline__ void store_digits(__half* dst, unsigned long long ua,
 template <typename In>
 __global__ void __launch_bounds__(kThr, 2)
 k_syrk_digits(const In* __restrict__ cube, int64_t N, int B, int parts,
-              const unsigned* __restrict__ ext, float* __restrict__ shift_out,
+              unsigned* __restrict__ ext, unsigned lost_max, float* __restrict__ shift_out,
               double* __restrict__ s1_part, double* __restrict__ s2_part,
               DevHeader* __restrict__ hdr) {
   extern __shared__ __align__(128) unsigned char smem[];
@@ -202,7 +216,9 @@ k_syrk_digits(const In* __restrict__ cube, int64_t N, int B, int parts,
     const float s = to_f32<In>(cube[b]);
     int k;
     if (!band_scale(ext[b], ext[B + b], s, &k)) bad = 1;
-    if (g == 0 && blockIdx.y == 0) shift_out[b] = s;
+    // the shift as it is subtracted, without its own lost bits
+    if (g == 0 && blockIdx.y == 0)
+      shift_out[b] = ext[b] == ~ext[B + b] ? s : ldexpf((float)to_fixed(s, k), -k);
   }
   if (tid < 2 * kTile) {
     const int h = tid >> 6, p = tid & 63;         // block, position in it
@@ -281,6 +297,7 @@ k_syrk_digits(const In* __restrict__ cube, int64_t N, int B, int parts,
         }
     ex_off = 0;
   };
+  unsigned lost[2] = {0u, 0u};     // values with lost bits, bands lane and lane + 32 (diagonal tiles)
   int par = 0, since = 0;
   for (int64_t c = n0; c < n1; c += kPx, par ^= 1) {
     asm volatile("cp.async.wait_all;" ::: "memory");
@@ -300,6 +317,10 @@ k_syrk_digits(const In* __restrict__ cube, int64_t N, int B, int parts,
           const int skip = (int)((((c + p) * B + b0) * (int64_t)sizeof(In)) & 15);
           const In* row = reinterpret_cast<const In*>(raw + (h * kPx + p) * raw_row<In>() + skip) + lane;
           const float va = inA ? to_f32<In>(row[0]) : 0.f, vb = inB ? to_f32<In>(row[32]) : 0.f;
+          if (diag) {
+            lost[0] += loses_bits(va, kA);
+            lost[1] += loses_bits(vb, kB);
+          }
           ua += (unsigned long long)(to_fixed(va, kA) - qA);
           ub += (unsigned long long)(to_fixed(vb, kB) - qB);
         }
@@ -401,6 +422,14 @@ k_syrk_digits(const In* __restrict__ cube, int64_t N, int B, int parts,
     }
   }
 
+  // a band of one value has none: its deviations are zero
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int b = ti * kTile + lane + 32 * h;
+    if (lost[h] != 0 && ext[b] != ~ext[B + b] && atomicAdd(&ext[2 * B + b], lost[h]) + lost[h] > lost_max)
+      hdr->fx_range = 1;
+  }
+
   if (ex_used) carry_ex();
   // pair sums, in units of 2^(-k_a - k_b); a sum with the constant band is S1
   const int s2_elems = B * (B + 1) / 2;
@@ -436,7 +465,7 @@ template <typename In>
 cudaError_t digits_typed(const In* cube, int64_t N, int B, float* shift, double* s1_part,
                          double* s2_part, int parts, unsigned* ext, DevHeader* hdr,
                          cudaStream_t st) {
-  cudaError_t e = cudaMemsetAsync(ext, 0, sizeof(unsigned) * 2 * B, st);
+  cudaError_t e = cudaMemsetAsync(ext, 0, sizeof(unsigned) * 3 * B, st);
   if (e != cudaSuccess) return e;
   const int grid = (int)std::min<int64_t>(4 * device_sms(), (N + 31) / 32);
   k_band_range<In><<<grid, 256, 0, st>>>(cube, N, B, ext);
@@ -446,8 +475,9 @@ cudaError_t digits_typed(const In* cube, int64_t N, int B, float* shift, double*
   e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   const int nb = (B + kTile) / kTile;
+  const unsigned lost_max = (unsigned)std::max<int64_t>(16, N >> 12);
   return launch_after(kern, dim3(parts, nb * (nb + 1) / 2), kThr, smem, st, cube, N, B, parts, ext,
-                      shift, s1_part, s2_part, hdr);
+                      lost_max, shift, s1_part, s2_part, hdr);
 }
 
 }  // namespace

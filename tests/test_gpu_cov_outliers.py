@@ -48,3 +48,42 @@ def test_p64_covariance_with_outliers_in_every_chunk(gbpca_lib):
     Y = (r.uniform(0.0, 1.0, (N, 3)) * np.exp2(r.integers(-13, 1, (N, 3)))).astype(np.float32)
     Y[0] = 0.25
     _check(gbpca_lib.covariance(torch.from_numpy(Y).cuda(), "p64"), Y)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("big", [2.0 ** 30, 2.0 ** 45, 2.0 ** 54, 9.96921e36])
+def test_p64_covariance_far_below_an_outlier(gbpca_lib, big):
+    """One fill value in band 0, where band 1 equals the shift: their covariance is that
+    of the other pixels, each entry to FP64."""
+    N = 8192
+    r = np.random.default_rng(7)
+    half = r.uniform(0.0, 0.25, (N // 2 - 1, 2)).astype(np.float32)
+    half[:, 1] = half[:, 0] * np.float32(0.5)
+    Y = np.full((N, 2), 0.5, dtype=np.float32)
+    Y[1:N // 2] += half                 # band 1's values are symmetric about the shift:
+    Y[N // 2:N - 1] = 1.0 - Y[1:N // 2]   # its mean is the shift, so nothing cancels
+    Y[N - 1, 0] = big
+    _, C, info = gbpca_lib.covariance(torch.from_numpy(Y).cuda(), "p64")
+    X = Y.astype(np.longdouble) - np.longdouble(0.5)
+    assert info["status"] == 0 and X[:, 1].sum() == 0
+    # FP64 sums of N terms (32 slots of 256 pixels)
+    bound = (256 + 32) * 2.0 ** -53 * (np.abs(X[:, 0]) * np.abs(X[:, 1])).sum() / (N - 1)
+    assert abs(np.longdouble(C[0, 1].item()) - (X[:, 0] * X[:, 1]).sum() / (N - 1)) <= bound
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("count", [3, 16, 17, 200])
+def test_p64_covariance_with_values_near_zero(gbpca_lib, count):
+    """A few values, or more than are let pass, with bits below the fixed point's unit."""
+    N = 40_000
+    r = np.random.default_rng(count)
+    Y = r.uniform(0.5, 1.0, (N, 3)).astype(np.float32)
+    Y[0] = 0.75
+    Y[7] = 60_000.0
+    Y[r.permutation(np.arange(8, N))[:count], 1] = r.uniform(1e-9, 1e-6, count)
+    mu, C, info = gbpca_lib.covariance(torch.from_numpy(Y).cuda(), "p64")
+    m, ref, sq = _moments(Y)
+    # FP64 sums of 256 pixels beside the roundings of _check, and 2^-52 sqrt(2 x 16)
+    bound = (256 + 64 + 12) * 2.0 ** -53 * np.sqrt(np.outer(sq, sq)) / (N - 1)
+    assert info["status"] == 0
+    assert np.all(np.abs(C.cpu().numpy() - ref) <= bound)
