@@ -130,7 +130,10 @@ __device__ __forceinline__ bool band_scale(unsigned max_o, unsigned min_o, float
     return false;
   const double d = fmax((double)top - (double)s, (double)s - (double)bot);
   const double a = fmax(fabs((double)top), fabs((double)bot));
-  if (d == 0.0) return true;                     // every digit is zero
+  if (d == 0.0) {                                // every digit is zero
+    if (a != 0.0) *k = min(60 - ilogb(a), 120);
+    return true;
+  }
   const int e = min(53 - ilogb(d), 60 - ilogb(a));
   if (e > 120) return false;
   *k = e;

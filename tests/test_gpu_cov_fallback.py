@@ -32,3 +32,18 @@ def test_workspace_of_more_bands_serves_fewer(gbpca_lib):
         ev = g.fit(Y, 4, precision="p64", workspace=ws)[1]
         ref = torch.linalg.eigvalsh(C).flip(0)
         assert (ev - ref).abs().max().item() <= 1e-10 * ref[0].item()
+
+
+@pytest.mark.gpu
+def test_constant_bands_of_every_size(gbpca_lib):
+    """A band of one value has a fixed-point form whatever the value (a fill value of 1e37 and
+    beyond as well): zero covariances, the value as its mean."""
+    values = (0.0, 3.25, -1e37, 9.96921e36, 3.4e38, 2.0 ** 63, 1e-30, -1e-39)
+    Y = np.random.default_rng(2).uniform(0.0, 1.0, (5000, len(values) + 2)).astype(np.float32)
+    Y[:, :len(values)] = values
+    mu, C, info = gbpca_lib.covariance(torch.from_numpy(Y).cuda(), "p64")
+    assert info["status"] == 0
+    assert np.array_equal(mu.cpu().numpy()[:len(values)], Y[0, :len(values)].astype(np.float64))
+    assert not C[:len(values)].any()
+    ref = np.cov(Y[:, len(values):].astype(np.float64).T)
+    assert np.abs(C[len(values):, len(values):].cpu().numpy() - ref).max() <= 1e-14
