@@ -91,8 +91,10 @@ typedef struct {
   double off_rel;    /* off(A)/||A||_F when the FP32 Jacobi stopped            */
   double tol_used;   /* the stop threshold the FP32 Jacobi applied             */
   double refine_res; /* largest |E_ij| of the last refinement correction (0 if none) */
-  int cov_fallback;  /* MIX only: 1 if a scaled value left the FP16 range and the
-                        covariance was recomputed in FP32 on the SIMT cores     */
+  int cov_fallback;  /* MIX: 1 if a scaled value left the FP16 range and the
+                        covariance was recomputed in FP32 on the SIMT cores;
+                        pca_covariance in P64: 1 if a band has no fixed-point
+                        form that holds its values and all was added in FP64   */
   int proj_fallback; /* MIX only: the same for the tensor-core projection       */
 } pca_info;
 
@@ -148,7 +150,8 @@ int pca_fit(const void *cube, pca_dtype dtype, int64_t N, int B, int k, double t
  *   first pixel's; where more than max(16, N / 4096) values of a band have
  *   bits below it, or a band has no such form, all is added in FP64 as in a
  *   fit; the bits cut off change C_ab by less than
- *   2^-52 sqrt(2 max(16, N / 4096)) sqrt(C_aa C_bb).  P32: FP32 SIMT; MIX:
+ *   2^-52 sqrt(2 max(16, N / 4096)) sqrt(C_aa C_bb); pca_info.cov_fallback
+ *   says which.  P32: FP32 SIMT; MIX:
  *   split-FP16 tensor cores on per-band shifted and power-of-two scaled values).
  * pca_eigh -- Algorithm 1 stage 4 on a given symmetric matrix A [B][B] FP64
  *   (device): cyclic Jacobi (Eqs. 2-10), FP64 refinement (P32: none; MIX: one

@@ -211,7 +211,7 @@ int pca_read_info(const void* workspace, void* stream, pca_info* info) {
   info->off_rel = h.off_rel;
   info->tol_used = h.tol_used;
   info->refine_res = h.refine_res;
-  info->cov_fallback = h.cov_range != 0 ? 1 : 0;
+  info->cov_fallback = (h.cov_range | h.fx_range) != 0 ? 1 : 0;
   info->proj_fallback = h.proj_range != 0 ? 1 : 0;
   return info->status;
 }

@@ -47,3 +47,25 @@ def test_constant_bands_of_every_size(gbpca_lib):
     assert not C[:len(values)].any()
     ref = np.cov(Y[:, len(values):].astype(np.float64).T)
     assert np.abs(C[len(values):, len(values):].cpu().numpy() - ref).max() <= 1e-14
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("kind,fallback", [("plain", 0), ("no-data pixel", 0), ("constant band", 0),
+                                           ("tiny spread", 1), ("fill value", 1), ("infinity", 1)])
+def test_p64_covariance_reports_its_form(gbpca_lib, kind, fallback):
+    Y = np.random.default_rng(3).uniform(0.0, 1.0, (50_000, 40)).astype(np.float32)
+    if kind == "no-data pixel":
+        Y[123] = -9999.0
+    elif kind == "constant band":
+        Y[:, 7] = 9.96921e36
+    elif kind == "tiny spread":
+        Y[:, 7] *= np.float32(1e-30)
+    elif kind == "fill value":
+        Y[123] = 9.96921e36
+    elif kind == "infinity":
+        Y[123, 7] = np.inf
+    _, _, info = gbpca_lib.covariance(torch.from_numpy(Y).cuda(), "p64")
+    assert info["status"] == (3 if kind == "infinity" else 0)
+    assert info["cov_fallback"] == fallback
+    # a fit adds in FP64 by itself
+    assert gbpca_lib.fit(torch.from_numpy(Y).cuda(), 1, precision="p64")[4]["cov_fallback"] == 0
