@@ -54,6 +54,7 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <cstddef>
 #include <type_traits>
 
 #include "jacobi.cuh"
@@ -77,7 +78,7 @@ constexpr int kSlots = 4;
 constexpr int kRecs = 128;        // records per slot: 32 lanes x W/2 pairs, W <= 8
 constexpr uint32_t kNone = 0xffffffffu;
 
-struct alignas(kJacobiParamsBytes) Params {
+struct ParamFields {
   const double* C;
   int B;
   float tol32;
@@ -89,6 +90,11 @@ struct alignas(kJacobiParamsBytes) Params {
   float* v32;
   DevHeader* hdr;
 };
+// An entry of a list: padded, not over-aligned (the host keeps lists in byte vectors).
+struct Params : ParamFields {
+  unsigned char pad[kJacobiParamsBytes - sizeof(ParamFields)];
+};
+static_assert(sizeof(Params) == kJacobiParamsBytes && alignof(Params) <= alignof(std::max_align_t));
 
 // pair_record (jacobi.cuh) with the drop test before the root.  The same values;
 // which one is faster depends on how the rest of the step is compiled: with

@@ -46,6 +46,7 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <cstddef>
 #include <type_traits>
 
 #include "jacobi.cuh"
@@ -59,7 +60,7 @@ namespace {
 constexpr int kMsg = 8;           // steps per record message (even)
 constexpr int kRing = 4;          // messages in flight to the vector CTAs
 
-struct alignas(kJacobiParamsBytes) Params {
+struct ParamFields {
   const double* C;
   int B;
   float tol32;
@@ -70,6 +71,11 @@ struct alignas(kJacobiParamsBytes) Params {
   float* v32;
   DevHeader* hdr;
 };
+// An entry of a list: padded, not over-aligned (the host keeps lists in byte vectors).
+struct Params : ParamFields {
+  unsigned char pad[kJacobiParamsBytes - sizeof(ParamFields)];
+};
+static_assert(sizeof(Params) == kJacobiParamsBytes && alignof(Params) <= alignof(std::max_align_t));
 
 struct Shared {
   uint64_t vfree[kRing];  // matrix CTA: its vector CTAs are done with a message
