@@ -18,9 +18,12 @@ oracle.  The same line carries the scene-shaped cubes (610x340x103 and
 synchronisations); `two_in_flight` gives the same fits two at a time on two
 streams, and `e2e` the fits of a stream of host-resident cubes through
 pca_fit_host with two calls in flight (with the one-at-a-time figure beside
-it), every step copying its cube in and its results out.
+it), every step copying its cube in and its results out.  The line stays below
+LINE_CHARS characters, with a few figures of each workload; --record FILE
+writes everything that was measured.
 
     python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
+                    [--record FILE]
 
 With torchrun (N > 1) every rank fits its own copy of the workload (weak
 scaling, no data-path collective); the step time is the max over ranks.
@@ -51,6 +54,7 @@ SM_LANES_FP32 = 128          # FP32 lanes per SM (sm_103a)
 NUM_SMS = 152
 C2_SIDE, C2_BANDS, C2_K = 2048, 224, 20
 ORACLE_SAMPLE_PIXELS = 1 << 18   # the oracle's bounded sample of the 2048^2 cube
+LINE_CHARS = 2500            # longest JSON line: what reads it may keep no more of the output
 
 
 def parse_args(argv=None):
@@ -60,6 +64,8 @@ def parse_args(argv=None):
     ap.add_argument("--warmup", type=int, default=5)
     ap.add_argument("--impl", choices=["ours", "reference"], default="ours")
     ap.add_argument("--precision", default="mix")
+    ap.add_argument("--record", metavar="FILE",
+                    help="also write everything measured to FILE (JSON)")
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--no-e2e", action="store_true")
     ap.add_argument("--no-batched", action="store_true",
@@ -1142,6 +1148,60 @@ def oracle_timings(args):
     return out
 
 
+# ------------------------------------------------------------------ the line
+def _short(x, digits=4):
+    """x with its floats rounded to so many significant digits."""
+    if isinstance(x, dict):
+        return {k: _short(v, digits) for k, v in x.items()}
+    if isinstance(x, (list, tuple)):
+        return [_short(v, digits) for v in x]
+    return float(f"{x:.{digits}g}") if isinstance(x, float) else x
+
+
+def _pick(d, *keys):
+    return {k: d[k] for k in keys if k in d}
+
+
+def summary_line(rec):
+    """The JSON line of a full record: the headline, its end-to-end figure, clocks and
+    bounds, and per workload the time of each form; groups are left out from the last
+    on where the line would be longer than LINE_CHARS."""
+    line = _pick(rec, "metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step",
+                 "higher_is_better", "scaling", "vs_baseline", "dtype", "data", "config")
+    if rec.get("e2e"):
+        line["e2e"] = _pick(rec["e2e"], "value", "unit", "h2d_bytes_per_step",
+                            "d2h_bytes_per_step", "ms_per_step", "one_in_flight_value")
+    line["gpu_launches"] = rec["gpu_launches"]
+    line["clocks"] = _pick(rec["clocks"], "sm_mhz", "sm_max_mhz", "reasons")
+    groups = {}
+    groups["forms_ms"] = {p: f["ms"] for p, f in (rec.get("forms") or {}).items()}
+    groups["stage_ms"] = {k: v for k, v in (rec.get("stage_ms_per_step") or {}).items()
+                          if k != "empty"}
+    if rec.get("roofline"):
+        groups["roofline"] = _pick(rec["roofline"], "kernel", "bound", "achieved", "peak", "unit",
+                                   "frac")
+    groups["hbm_frac"] = {k: v["frac"] for k, v in (rec.get("hbm_kernels") or {}).items()}
+    groups["eig_rel_err"] = {k: v["eig_rel_err_topk_max"] for k, v in (rec.get("errors") or {}).items()
+                             if "eig_rel_err_topk_max" in v}
+    if rec.get("cpu_baseline"):
+        groups["cpu_baseline"] = _pick(rec["cpu_baseline"], "value", "unit", "cores", "kind")
+    groups["two_in_flight_ms"] = {k: v["ms_per_fit"] for k, v in (rec.get("two_in_flight") or {}).items()
+                                  if isinstance(v, dict) and "ms_per_fit" in v}
+    for key, name, ms in (("batched", "batched_256_tiles_ms", "ms"),
+                          ("scenes", "scenes_ms", "ms_per_step"),
+                          ("mixing_100x100x128", "mixing_100x100x128_ms", "ms")):
+        if rec.get(key):
+            groups[name] = {p: f[ms] for p, f in rec[key]["forms"].items()}
+    if rec.get("differentiation"):
+        groups["differentiation"] = _pick(rec["differentiation"], "forward_ms", "backward_ms")
+    groups["paper_shapes_k1_mix_ms"] = {s["workload"]: s["mix"]["ms"]
+                                        for s in rec.get("paper_shapes_k1") or []}
+    for name, group in groups.items():
+        if group and len(json.dumps({**line, name: _short(group)})) <= LINE_CHARS:
+            line[name] = _short(group)
+    return line
+
+
 # ------------------------------------------------------------------ our arm
 def main(argv=None):
     args = parse_args(argv)
@@ -1236,29 +1296,32 @@ def main(argv=None):
 
     launches = g.kernel_launches(args.precision, c2["k"]) * args.steps
     forms = c2["forms"]
-    line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
-            "warmup": args.warmup, "ms_per_step": t_head / args.steps * 1e3,
-            "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
-            "dtype": ("bf16 in; f16 tensor products (x1, x3 when a lo part is non-zero), f32 "
-                      "accumulation; f32 Jacobi; f64/double-float refinement"
-                      if args.precision == "mix" else args.precision),
-            "data": "synthetic",
-            "config": {"workload": WORKLOAD, "precision": args.precision,
-                       "cube": f"N={c2['N']} B={c2['B']} bf16 (drawn on the device)",
-                       "k": c2["k"], "units_per_step": c2["units"],
-                       "l2": "input (1.88 GB) larger than L2; no flush",
-                       "parallelism": f"replicas x{world}" if world > 1 else "1 GPU"},
-            "forms": forms, "stage_ms_per_step": forms[args.precision]["stage_ms"],
-            "hbm_kernels": c2["hbm"], "errors": c2["errors"], "roofline": roof,
-            "step_hbm_frac": (2 * c2["N"] * c2["B"] * 2 + 4 * c2["N"] * c2["k"])
-            / (t_head / args.steps) / 1e9 / peaks["hbm_gbs"],
-            "cpu_baseline": cpu, "oracle_timings": timings, "e2e": c2["e2e"],
-            "two_in_flight": c2.get("two_in_flight"),
-            "gpu_launches": launches, "clocks": sampler.summary(),
-            "scenes": scenes, "mixing_100x100x128": c0, "differentiation": diff,
-            "batched": batched, "paper_shapes_k1": shapes}
+    record = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
+              "warmup": args.warmup, "ms_per_step": t_head / args.steps * 1e3,
+              "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
+              "dtype": ("bf16 in; f16 tensor products (x1, x3 when a lo part is non-zero), f32 "
+                        "accumulation; f32 Jacobi; f64/double-float refinement"
+                        if args.precision == "mix" else args.precision),
+              "data": "synthetic",
+              "config": {"workload": WORKLOAD, "precision": args.precision,
+                         "cube": f"N={c2['N']} B={c2['B']} bf16 (drawn on the device)",
+                         "k": c2["k"], "units_per_step": c2["units"],
+                         "l2": "input (1.88 GB) larger than L2; no flush",
+                         "parallelism": f"replicas x{world}" if world > 1 else "1 GPU"},
+              "forms": forms, "stage_ms_per_step": forms[args.precision]["stage_ms"],
+              "hbm_kernels": c2["hbm"], "errors": c2["errors"], "roofline": roof,
+              "step_hbm_frac": (2 * c2["N"] * c2["B"] * 2 + 4 * c2["N"] * c2["k"])
+              / (t_head / args.steps) / 1e9 / peaks["hbm_gbs"],
+              "cpu_baseline": cpu, "oracle_timings": timings, "e2e": c2["e2e"],
+              "two_in_flight": c2.get("two_in_flight"),
+              "gpu_launches": launches, "clocks": sampler.summary(),
+              "scenes": scenes, "mixing_100x100x128": c0, "differentiation": diff,
+              "batched": batched, "paper_shapes_k1": shapes}
     if rank == 0:
-        print(json.dumps(line))
+        if args.record:
+            with open(args.record, "w") as f:
+                json.dump(record, f)
+        print(json.dumps(summary_line(record)))
     if world > 1:
         import torch.distributed as dist
         dist.destroy_process_group()
