@@ -200,7 +200,7 @@ cudaError_t launch_jacobi_cluster(const double* C, int B, float tol32, int sweep
                                   cudaStream_t st);
 
 // CTAs (= SMs) the cluster Jacobi uses for B bands: nA matrix CTAs + nV V CTAs.
-bool jacobi_cluster_shape(int B, int* nA, int* nV);
+void jacobi_cluster_shape(int B, int* nA, int* nV);
 
 // Drops the padding slot: lam (FP64) [B] and Vc [B][B] in slot order, Vc as
 // double-float (hi, lo) pairs.

@@ -31,32 +31,43 @@ __device__ __forceinline__ float sqrt_est(float x) {
 // reciprocal/root steps instead of four (the step's critical path runs
 // through this record).  Where d^2 + n^2 could leave the FP32 range (|d| or
 // |n| beyond 1e18, or both below 1e-18) the scale-free tau form is taken.
-// Here the drop test runs beside the root, not before it (k_jacobi_cluster.cu has
-// the other form too).
+// The drop test runs beside the root, and one rotation follows either root.  With the
+// test before the root and a rotation for each in the cluster kernel (the same values) a step
+// takes, in us: 144 bands 0.757 for 0.762 here, 188 bands 0.810 / 0.795, 224 bands 0.817 /
+// 0.805, 246 bands 0.846 / 0.837, 252 bands 0.881 / 0.894, 256 bands 0.900 / 0.910; the Jacobi
+// stage of 256 tiles 7.2 to 7.7 ms in both.
 __device__ __forceinline__ float4 pair_record(float app, float aqq, float apq) {
   const float thr = 5.9604645e-08f * sqrt_est(fabsf(app)) * sqrt_est(fabsf(aqq));
+  const bool keep = fabsf(apq) > thr;
   const float d = aqq - app, n = 2.f * apq;
   const float ad = fabsf(d), an = fabsf(n);
-  const bool keep = fabsf(apq) > thr;
-  float tt;
-  if (!keep || (ad < 1e18f && an < 1e18f && (ad > 1e-18f || an > 1e-18f))) {
+  auto root = [&]() {
     const float q = fmaf(d, d, n * n);
-    tt = an * rcp_nr(ad + q * rsqrt_nr(q));
-    tt = (d != 0.f && ((d < 0.f) != (n < 0.f))) ? -tt : tt;
-  } else {
+    const float t = an * rcp_nr(ad + q * rsqrt_nr(q));
+    return (d != 0.f && ((d < 0.f) != (n < 0.f))) ? -t : t;
+  };
+  auto root_scale_free = [&]() {
     const float tau = (aqq - app) * rcp_nr(2.f * apq);
     const float at = fabsf(tau);
+    float t;
     if (at > 1e18f) {
-      tt = 0.5f * rcp_nr(at);
+      t = 0.5f * rcp_nr(at);
     } else {
       const float u = fmaf(tau, tau, 1.f);
-      tt = rcp_nr(at + u * rsqrt_nr(u));
+      t = rcp_nr(at + u * rsqrt_nr(u));
     }
-    tt = (tau >= 0.f) ? tt : -tt;
-  }
-  const float c = rsqrt_nr(fmaf(tt, tt, 1.f));
-  return keep ? make_float4(c, tt * c, fmaf(tt, apq, aqq), fmaf(-tt, apq, app))
-              : make_float4(1.f, 0.f, aqq, app);
+    return (tau >= 0.f) ? t : -t;
+  };
+  auto rotation = [&](float t) {
+    const float c = rsqrt_nr(fmaf(t, t, 1.f));
+    return make_float4(c, t * c, fmaf(t, apq, aqq), fmaf(-t, apq, app));
+  };
+  const bool in_range = ad < 1e18f && an < 1e18f && (ad > 1e-18f || an > 1e-18f);
+  float t;
+  if (!keep || in_range) t = root();
+  else t = root_scale_free();
+  const float4 r = rotation(t);
+  return keep ? r : make_float4(1.f, 0.f, aqq, app);
 }
 
 // M' = G_I M G_J, G = [[s, c], [c, -s]].

@@ -75,7 +75,8 @@ constexpr int kWideVRows = 3;     // the same for the fewer-CTA variant
 constexpr int kWideItems = 3;
 constexpr int kMaxCl = 8;
 constexpr int kSlots = 4;
-constexpr int kRecs = 128;        // records per slot: 32 lanes x W/2 pairs, W <= 8
+constexpr int kWidth = 8;         // W: positions of a V row per lane (256 bands over 32 lanes)
+constexpr int kRecs = 32 * kWidth / 2;   // records per slot
 constexpr uint32_t kNone = 0xffffffffu;
 
 struct ParamFields {
@@ -95,41 +96,6 @@ struct Params : ParamFields {
   unsigned char pad[kJacobiParamsBytes - sizeof(ParamFields)];
 };
 static_assert(sizeof(Params) == kJacobiParamsBytes && alignof(Params) <= alignof(std::max_align_t));
-
-// pair_record (jacobi.cuh) with the drop test before the root.  The same values;
-// which one is faster depends on how the rest of the step is compiled: with
-// 224 bands 0.825 us a step with the test first, 0.811 beside
-// (188 bands 0.82 / 0.80), with 256 bands 0.905 / 0.918 -- so the test goes first
-// above 224 bands, and in the wide variant (the Jacobi stage of the 256-tile
-// batch 7.5 ms, 8.5 with the test beside).
-__device__ __forceinline__ float4 pair_record_drop_first(float app, float aqq, float apq) {
-  const float thr = 5.9604645e-08f * sqrt_est(fabsf(app)) * sqrt_est(fabsf(aqq));
-  if (!(fabsf(apq) > thr)) return make_float4(1.f, 0.f, aqq, app);
-  {
-    const float d = aqq - app, n = 2.f * apq;
-    const float ad = fabsf(d), an = fabsf(n);
-    if (ad < 1e18f && an < 1e18f && (ad > 1e-18f || an > 1e-18f)) {
-      const float q = fmaf(d, d, n * n);
-      float tt = an * rcp_nr(ad + q * rsqrt_nr(q));
-      tt = (d != 0.f && ((d < 0.f) != (n < 0.f))) ? -tt : tt;
-      const float c = rsqrt_nr(fmaf(tt, tt, 1.f));
-      return make_float4(c, tt * c, fmaf(tt, apq, aqq), fmaf(-tt, apq, app));
-    }
-  }
-  const float tau = (aqq - app) * rcp_nr(2.f * apq);
-  const float at = fabsf(tau);
-  float tt;
-  if (at > 1e18f) {
-    tt = 0.5f * rcp_nr(at);
-  } else {
-    const float u = fmaf(tau, tau, 1.f);
-    tt = rcp_nr(at + u * rsqrt_nr(u));
-  }
-  tt = (tau >= 0.f) ? tt : -tt;
-  const float c = rsqrt_nr(fmaf(tt, tt, 1.f));
-  return make_float4(c, tt * c, fmaf(tt, apq, aqq), fmaf(-tt, apq, app));
-}
-
 
 struct Shared {
   uint64_t mbar[kSlots];  // step s+1 completes on mbar[(s + 1) % kSlots]
@@ -236,13 +202,10 @@ __device__ __forceinline__ const Params& par(const Params& one, const Params* li
 
 // One matrix per cluster: `one` when list is null, else list[cluster index]
 // (every entry of a list has the cluster size one.nA).
-template <int W, int VR, int MI, bool kDropFirst>
+template <int VR, int MI>
 __global__ void __launch_bounds__(kThreads, 1)
 k_jacobi_cluster(const __grid_constant__ Params one, const Params* __restrict__ list) {
-  constexpr int H = W / 2;                 // pairs per lane in a V row
-  auto record = [](float app, float aqq, float apq) {
-    return kDropFirst ? pair_record_drop_first(app, aqq, apq) : pair_record(app, aqq, apq);
-  };
+  constexpr int W = kWidth, H = W / 2;     // positions and pairs per lane in a V row
   extern __shared__ __align__(16) float rows[];
   __shared__ Shared sh;
   cg::cluster_group cl = cg::this_cluster();
@@ -479,7 +442,7 @@ k_jacobi_cluster(const __grid_constant__ Params one, const Params* __restrict__ 
     if (tid < I_hi - I_lo) {
       const int I = I_lo + tid, p = 2 * I;
       float* apq = rows + (p - R0) * Bp + p + 1;
-      push_record<H>(cl, &sh, ncl, gs % kSlots, I, record(sh.dg[p], sh.dg[p + 1], *apq));
+      push_record<H>(cl, &sh, ncl, gs % kSlots, I, pair_record(sh.dg[p], sh.dg[p + 1], *apq));
       *apq = 0.f;
       if (I == I_lo && has_prev) cl.map_shared_rank(rows, rank - 1)[(size_t)halo_row * Bp + p + 1] = 0.f;
     }
@@ -515,7 +478,7 @@ k_jacobi_cluster(const __grid_constant__ Params one, const Params* __restrict__ 
           const float4 gI = rec4<H>(&sh, cur, I), gJ = rec4<H>(&sh, cur, I + 1);
           rot_block(make_float2(gI.x, gI.y), make_float2(gJ.x, gJ.y), m00, m01, m10, m11);
           if (!last) {  // (q_I, p_{I+1}) is the off-diagonal of a next-step pair
-            push_record_async<H>(&sh, ncl, nxt, e == 0 ? I : I + 1, record(gI.w, gJ.z, m10));
+            push_record_async<H>(&sh, ncl, nxt, e == 0 ? I : I + 1, pair_record(gI.w, gJ.z, m10));
             m10 = 0.f;
           }
           if (e == 0) {
@@ -541,7 +504,7 @@ k_jacobi_cluster(const __grid_constant__ Params one, const Params* __restrict__ 
             float n0 = fmaf(x, g.y, y * g.x);
             const float n1 = fmaf(x, g.x, -y * g.y);
             if (!last) {
-              push_record_async<H>(&sh, ncl, nxt, 0, record(sh.dd[prv][rix<H>(0)].x, g.z, n0));
+              push_record_async<H>(&sh, ncl, nxt, 0, pair_record(sh.dd[prv][rix<H>(0)].x, g.z, n0));
               n0 = 0.f;
             }
             a[0] = n0;
@@ -555,7 +518,7 @@ k_jacobi_cluster(const __grid_constant__ Params one, const Params* __restrict__ 
             float n1 = fmaf(g.x, x, -g.y * y);
             if (!last) {
               push_record_async<H>(&sh, ncl, nxt, P - 1,
-                                   record(g.w, sh.dd[prv][rix<H>(P - 1)].y, n1));
+                                   pair_record(g.w, sh.dd[prv][rix<H>(P - 1)].y, n1));
               n1 = 0.f;
             }
             a[0] = n0;
@@ -790,9 +753,7 @@ int fewest_ctas(int B, int n0) {
 cudaError_t launch_clusters(const Params& one, const Params* list, int count, size_t smem,
                             cudaStream_t st) {
   const bool wide = one.nA < min_ctas(one.B);
-  auto kern = wide ? k_jacobi_cluster<8, kWideVRows, kWideItems, true>
-              : round_even(one.B) > 224 ? k_jacobi_cluster<8, kVRows, kMaxItems, true>
-                                        : k_jacobi_cluster<8, kVRows, kMaxItems, false>;
+  auto kern = wide ? k_jacobi_cluster<kWideVRows, kWideItems> : k_jacobi_cluster<kVRows, kMaxItems>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
@@ -817,8 +778,8 @@ cudaError_t launch_clusters(const Params& one, const Params* list, int count, si
 // ------------------------------------------------ which kernel a matrix takes
 // Up to 128 bands k_jacobi_sm.cu, whose matrix stays in one SM; above, the one
 // of this file: its blocks are spread over up to 8 SMs, and one SM's shared memory
-// would take longer for them than the exchange between SMs does (128 bands: 0.70
-// us a step on one SM, 0.73 here; 160 bands: 1.0 against 0.80).
+// would take longer for them than the exchange between SMs does (128 bands: 0.69
+// us a step on one SM, 0.73 here; 160 bands: 1.0 against 0.79).
 
 int jacobi_width(int B) {
   const int Bp = round_even(B);
@@ -826,12 +787,11 @@ int jacobi_width(int B) {
 }
 
 // The latency-oriented shape of the single-matrix form.
-bool jacobi_cluster_shape(int B, int* nA, int* nV) {
+void jacobi_cluster_shape(int B, int* nA, int* nV) {
   const int Bp = round_even(B);
   const bool sm = jacobi_sm_supported(B);
   *nA = sm ? 1 : kMaxCl;
   *nV = sm ? (Bp <= 64 ? 1 : 3) : 0;
-  return true;
 }
 
 cudaError_t launch_jacobi_cluster(const double* C, int B, float tol32, int sweeps_max,

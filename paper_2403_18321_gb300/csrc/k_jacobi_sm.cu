@@ -34,12 +34,13 @@
 //     kRing messages.
 //
 // Per step (FP32 form, whole solve over its steps), against k_jacobi_cluster.cu on
-// 1 to 4 CTAs: 32 bands 0.36 us / 0.77, 64 bands 0.36 / 0.67, 100 bands 0.52 /
-// 0.69, 128 bands 0.70 / 0.73; same bits.  Tried and slower: the matrix over several
+// 1 to 4 CTAs: 32 bands 0.34 us / 0.77, 64 bands 0.33 / 0.67, 100 bands 0.51 /
+// 0.69, 128 bands 0.69 / 0.73; same bits.  Tried and slower: the matrix over several
 // CTAs that form every angle themselves and exchange bands and edge rows every four
-// steps (224 bands: 1.14 us against 0.82; the exchange takes 1.6 us), the matrix in
-// registers, 8 x 4 entries a lane (128 bands 0.66, 64 bands 0.46, 188 bands 1.14),
-// blocks one at a time (100 bands 0.58), 1024 threads (128 bands 0.75).
+// steps (224 bands: 1.14 us against 0.82; the exchange takes 1.6 us), blocks one at a
+// time (100 bands 0.58), 1024 threads (128 bands 0.75).  The matrix in registers, 8 x 4
+// entries a lane, was slower up to about 120 bands (64 bands 0.46) and above 128 (188 bands
+// 1.14) and a little faster at 128 (0.66): not worth a form of its own.
 //
 // Every mbarrier wait is bounded: a CTA that gives up stops waiting, and the
 // sweep's stop test ends the solve with PCA_ERR_TIMEOUT.
