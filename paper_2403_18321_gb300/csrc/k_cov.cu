@@ -47,8 +47,10 @@ __host__ __device__ inline int raw_units(int B, int el) { return (kStage * B * e
 // 0), band-tile group grp.  Each thread owns one TM x TN tile of the upper
 // block-triangle of S2 and adds its products pixel by pixel.
 //
-// Bound: the FP32 (FP64) pipe.  The pixels come in by asynchronous copies, one
-// stage ahead, and are centred once per CTA into a second buffer (loads into
+// Bound: the FP32 (FP64) pipe and issue while an SM works, and the last round of CTAs
+// (610 x 340 x 103 FP32: 320 CTAs, 304 resident, an SM active 54% of the launch; 2.6 of 4
+// instructions issued a cycle).  The pixels come in by asynchronous copies, up to three
+// stages ahead, and are centred once per CTA into a second buffer (loads into
 // registers, a few at a time between two barriers, took 14 of every 15 us).
 // Tile t holds TM / U units of U consecutive bands (16 bytes), unit u being
 // bands u Bu + U t and on, so that the lanes of a warp -- consecutive tiles of

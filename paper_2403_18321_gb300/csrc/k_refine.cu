@@ -15,7 +15,7 @@
 // non-orthogonal by O(||E||^2); a closing Newton-Schulz step
 // V <- V (3I - V^T V)/2 squares that away (launch_orthonormalize).
 //
-// Arithmetic: GB300 executes FP64 at about 1/58 of its FP32 rate (1.9 DFMA
+// Arithmetic: GB300 executes FP64 at 1/67 of its FP32 rate (1.9 DFMA of 128
 // per clock per SM), which would make each B^3 product cost ~20 us at
 // B = 224.  The products therefore run in double-float: every matrix is kept
 // as an unevaluated sum hi + lo of two FP32 values (48-bit significand), each

@@ -1,8 +1,8 @@
 // k_syrk_digits.cu -- partials of the P64 covariance call from exact integer
 // products on the tensor cores.
 //
-// FP64 runs at about 1/67 of the FP32 rate on this GPU (1.9 FMAs per clock and
-// SM), so that S2 = sum_n x_n x_n^T of 350 x 350 pixels of 188 bands costs
+// FP64 runs at 1/67 of the FP32 rate on this GPU (1.9 FMAs per clock and SM
+// against 128), so that S2 = sum_n x_n x_n^T of 350 x 350 pixels of 188 bands costs
 // 3.6 ms at its full rate.  Here x = y - s is held as a 56-bit fixed-point number per band
 // and written as seven signed 8-bit digits D_0 .. D_6 (splitting into slices whose
 // products are exact: Ozaki, Ogita, Oishi and Rump, Numer. Algorithms 59, 2012).
@@ -27,11 +27,11 @@
 // that sqrt(N / 2) 2^-57 at its worst (1.3e-15 at 16 values, 5e-15 at 10^6 pixels), and lets
 // the few values near zero of a cube with no-data pixels pass.
 //
-// The covariance call, FP64 products -> these: 350 x 350 x 188 FP32 4.74 -> 0.61 ms,
-// 610 x 340 x 103 2.88 -> 0.51, 512 x 512 x 224 BF16 13.7 -> 1.22, 10,000 x 50 0.189 -> 0.058.
-// Its error against extended precision, over cubes of 28,000 to 57,000 pixels and
-// 51 to 244 bands (relative to sqrt(C_aa C_bb), root mean square): FP64 products
-// 8e-17 .. 1.1e-15, these 9e-17 .. 1.4e-16.
+// The covariance call, FP64 products -> these: 350 x 350 x 188 FP32 4.74 -> 0.68 ms,
+// 610 x 340 x 103 2.88 -> 0.57, 512 x 512 x 224 BF16 13.7 -> 1.44, 10,000 x 50 0.189 -> 0.072.
+// Its error against extended precision, over cubes of 28,000 to 10^6 pixels and 24 to 244
+// bands, with and without a pixel of 300 to 65,535 among values of a lower range (relative to
+// sqrt(C_aa C_bb), root mean square): FP64 products 1.3e-16 .. 1.3e-14, these 9e-17 .. 2.8e-16.
 //
 // Band B of the tiles is a constant band whose only digit is D_0 = 64, so that its
 // products are the band sums S1.
@@ -189,11 +189,12 @@ __device__ __forceinline__ void store_digits(__half* dst, unsigned long long ua,
 }
 
 // Grid: x = partial slot (pixels N x / parts ..), y = tile of the upper block-triangle.
-// Bound: issue (half of the slots) and the latency of the shared-memory reads; the tensor
-// pipe is active 29% of the time, the ALU (conversion, digits) 55%.  A chunk's rows come by
+// Bound: issue (58% of the slots) and the latency of the shared-memory reads; the tensor
+// pipe is active 26% of the time, the ALU (conversion, digits) 58%.  A chunk's rows come by
 // asynchronous copies during the products of the one before, and 8 warps of 32 x 16 outputs
 // (128 registers) hide more latency than 4 of 32 x 32 (237): 350 x 350 x 188, with loads
-// into registers and 4 warps 1.02 ms, so 0.61.
+// into registers and 4 warps 1.02 ms, so 0.61 (levels 0 .. 7; 0.68 with all levels and the
+// count of lost bits).
 template <typename In>
 __global__ void __launch_bounds__(kThr, 2)
 k_syrk_digits(const In* __restrict__ cube, int64_t N, int B, int parts,
