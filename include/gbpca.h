@@ -147,7 +147,7 @@ int pca_fit(const void *cube, pca_dtype dtype, int64_t N, int B, int k, double t
  *   covariance form (P64: exact products and sums of fixed-point values,
  *   rounded to FP64 partials, where a fit adds in FP64.  The fixed point's
  *   unit is at most 2^-53 of the largest distance of a value from the
- *   first pixel's; where more than max(16, N / 4096) values of a band have
+ *   first pixel's (2^-52 above 2*10^10 pixels); where more than max(16, N / 4096) values of a band have
  *   bits below it, or a band has no such form, all is added in FP64 as in a
  *   fit; the bits cut off change C_ab by less than
  *   2^-52 sqrt(2 max(16, N / 4096)) sqrt(C_aa C_bb); pca_info.cov_fallback

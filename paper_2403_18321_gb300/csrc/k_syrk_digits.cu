@@ -21,7 +21,7 @@
 // or a spread too small for an FP32 scale sets hdr->fx_range, and the FP64 SIMT
 // form (guarded by it) does the work.  So does a band of which more than lost_max values have
 // bits below the scale's unit u, which is at most 2^-53 of the distance d of two of its
-// values (values below 2^-30 of the farthest one; their bits are cut off).  n such values
+// values (2^-52 in slots of more than 2^26 pixels).  n such values, below 2^-30 of the farthest one,
 // move a covariance by at most u sqrt(n) of sqrt(C_bb / (N - 1)), and C_aa (N - 1) >= d^2 / 2:
 // 2^-52 sqrt(2 n) of sqrt(C_aa C_bb) for both factors.  lost_max = N / 4096 (16 at least) makes
 // that sqrt(N / 2) 2^-57 at its worst (1.3e-15 at 16 values, 5e-15 at 10^6 pixels), and lets
@@ -33,8 +33,8 @@
 // bands, with and without a pixel of 300 to 65,535 among values of a lower range (relative to
 // sqrt(C_aa C_bb), root mean square): FP64 products 1.3e-16 .. 1.3e-14, these 9e-17 .. 2.8e-16.
 //
-// Band B of the tiles is a constant band whose only digit is D_0 = 64, so that its
-// products are the band sums S1.
+// Band B of the tiles is a constant band whose only digit is D_0, so that its products are
+// the band sums S1.
 //
 // mma.sync rather than tcgen05: the sums of a level leave the accumulators after every
 // 32 pixels, which in registers costs an FADD and an IMAD, while from TMEM they
@@ -118,11 +118,12 @@ k_band_range(const In* __restrict__ cube, int64_t N, int B, unsigned* __restrict
   }
 }
 
-// The scale 2^k of a band about its shift s: |x| 2^k < 2^54, and |y| 2^k < 2^61 (which only
-// bands whose values all lie within 2^-7 of each other reach: their digits then end at
+// The scale 2^k of a band about its shift s: |x| 2^k < 2^(top_bit + 1), and |y| 2^k < 2^61 (which
+// only bands whose values all lie within 2^-7 of each other reach: their digits then end at
 // D_2, so that nothing is left out).  False: no such scale (a non-finite value, or a spread
 // too small).
-__device__ __forceinline__ bool band_scale(unsigned max_o, unsigned min_o, float s, int* k) {
+__device__ __forceinline__ bool band_scale(unsigned max_o, unsigned min_o, float s, int top_bit,
+                                           int* k) {
   const float top = unordered(max_o), bot = unordered(~min_o);
   *k = 0;
   if (!(fabsf(top) <= 3.4028234e38f) || !(fabsf(bot) <= 3.4028234e38f) ||
@@ -134,7 +135,7 @@ __device__ __forceinline__ bool band_scale(unsigned max_o, unsigned min_o, float
     if (a != 0.0) *k = min(60 - ilogb(a), 120);
     return true;
   }
-  const int e = min(53 - ilogb(d), 60 - ilogb(a));
+  const int e = min(top_bit - ilogb(d), 60 - ilogb(a));
   if (e > 120) return false;
   *k = e;
   return true;
@@ -214,12 +215,15 @@ k_syrk_digits(const In* __restrict__ cube, int64_t N, int B, int parts,
   const bool diag = ti == tj;
   pdl_wait();
 
+  // |x| < 2^54, or 2^53 where a slot has more than 2^26 pixels (up to 2^28 in 280 GB): the
+  // sum of their squares, in units of 2^72, stays below 2^62
+  const int top_bit = N / parts >= (int64_t)1 << 26 ? 52 : 53;
   // every CTA looks at every band, so that all take the same way
   int bad = 0;
   for (int b = tid; b < B; b += kThr) {
     const float s = to_f32<In>(cube[b]);
     int k;
-    if (!band_scale(ext[b], ext[B + b], s, &k)) bad = 1;
+    if (!band_scale(ext[b], ext[B + b], s, top_bit, &k)) bad = 1;
     // the shift as it is subtracted, without its own lost bits
     if (g == 0 && blockIdx.y == 0)
       shift_out[b] = ext[b] == ~ext[B + b] ? s : ldexpf((float)to_fixed(s, k), -k);
@@ -227,14 +231,14 @@ k_syrk_digits(const In* __restrict__ cube, int64_t N, int B, int parts,
   if (tid < 2 * kTile) {
     const int h = tid >> 6, p = tid & 63;         // block, position in it
     const int b = (h ? tj : ti) * kTile + (p >> 1) + 32 * (p & 1);
-    int k = b == B ? 54 : 0;               // the constant band: D_0 = 64
+    int k = b == B ? top_bit + 1 : 0;      // the constant band: D_0 = 64 (32)
     long long q0 = 0;
     if (b < B) {
       const float s = to_f32<In>(cube[b]);
-      band_scale(ext[b], ext[B + b], s, &k);
+      band_scale(ext[b], ext[B + b], s, top_bit, &k);
       q0 = to_fixed(s, k);
     } else if (b == B) {
-      q0 = -(64ll << 48);                         // digits of 0 - q0
+      q0 = -(1ll << (top_bit + 1));               // digits of 0 - q0
     }
     sy->q0[h][p] = q0;
     sy->k[h][p] = k;
